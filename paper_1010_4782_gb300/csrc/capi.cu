@@ -7,6 +7,7 @@
 // CG state back only between blocks.  After Fig. 1 stops, the true residual
 // b - A x is recomputed with native FP64 arithmetic and Fig. 1 restarts from
 // the current x while it exceeds tol.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -122,7 +123,13 @@ void begin_call(stag_handle* h) {
     cuda_check(h, cudaStreamWaitEvent(h->s, h->ev_in, 0), "cudaStreamWaitEvent");
 }
 
-void end_call(stag_handle* h) { cuda_check(h, cudaStreamSynchronize(h->s), "cudaStreamSynchronize"); }
+void end_call(stag_handle* h) {
+    cuda_check(h, cudaStreamSynchronize(h->s), "cudaStreamSynchronize");
+    if (h->timeout_host && *static_cast<volatile int*>(h->timeout_host)) {
+        *h->timeout_host = 0;
+        fail(h, STAG_ERR_TIMEOUT, "a bounded wait between the blocks of a kernel ran out");
+    }
+}
 
 // long_recon = 12 accepts Naik links whose L / long_scale deviates from SU(3)
 // by at most this (entries of L^dag L / c^2 - 1, and det L / c^3 - 1): the third
@@ -307,8 +314,72 @@ void ensure_graph(stag_handle* h) {
     cuda_check(h, e, "graph instantiate");
 }
 
+// Most iterations of one launch of resident.cu (a few milliseconds, so that a
+// call never holds the GPU for long in one kernel).
+constexpr int kResidentIters = 512;
+
+// Is the iteration's arithmetic FP32 (the mixed-precision inner iteration)?
+bool iterates_in_fp32(const stag_handle* h) { return h->opt.inner != STAG_INNER_NONE; }
+
+void launch_resident(stag_handle* h, int iters) {
+    const Geom& g = h->g;
+    ResidentWork w = h->rwork;
+    if (!h->opt.timing) w.ns = nullptr;
+    cudaError_t e;
+    if (iterates_in_fp32(h)) {
+        LoLinks L;
+        L.fat32 = h->fat32;
+        L.lng32 = h->lng32;
+        L.fat16 = h->fat16;
+        L.lng16 = h->lng16;
+        L.fatb16 = h->fatb16;
+        L.lngb16 = h->lngb16;
+        L.two_row_fat = h->opt.link_recon == 12;
+        L.vectors32 = h->opt.inner == STAG_INNER_F32_L16;
+        L.lng_inv_scale = lo_long_inv_scale(h);
+        e = launch_resident_lo(g, L, h->lo_d, h->lo_t, h->lo_r, h->lo_y, h->scal, w, iters, h->s);
+    } else if (use_ff(h)) {
+        e = launch_resident_ff(g, links(h), static_cast<float4*>(h->d), static_cast<float4*>(h->t),
+                               reinterpret_cast<float4*>(h->r), h->x, h->scal, w, iters, h->opt.check_interval, h->s);
+    } else {
+        e = launch_resident_f64(g, links(h), static_cast<double2*>(h->d), static_cast<double2*>(h->t), h->r, h->x,
+                                h->scal, w, iters, h->s);
+    }
+    cuda_check(h, e, "resident CG launch");
+    h->launches += 1;
+}
+
+// Fig. 1 in launches of many iterations each (resident.cu).  A block hook is
+// called every check_interval iterations, as with blocks of launches.
+void run_fig1_resident(stag_handle* h) {
+    const int K = h->opt.check_interval;
+    const int iters = h->block_hook ? K : std::max(1, kResidentIters / K) * K;
+    long long iter_before = 0;  // a run starts at iteration 0
+    do {
+        launch_resident(h, iters);
+        read_state(h);
+        if (h->block_hook) h->block_hook();
+        if (h->opt.timing) {
+            unsigned long long ns[4];
+            cuda_check(h, cudaMemcpyAsync(ns, h->rwork.ns, sizeof(ns), cudaMemcpyDeviceToHost, h->s), "read times");
+            cuda_check(h, cudaMemsetAsync(h->rwork.ns, 0, sizeof(ns), h->s), "clear times");
+            end_call(h);
+            const long long active = h->scal_host->iter - iter_before;
+            for (int j = 0; j < STAG_KERNEL_COUNT; ++j) {
+                h->stats[j].ms += 1e-6 * (double)ns[j];
+                h->stats[j].launches += j == 3 && h->scal_host->done && active > 0 ? active - 1 : active;
+            }
+        }
+        iter_before = h->scal_host->iter;
+    } while (!h->scal_host->done);
+}
+
 // Runs Fig. 1 from the state prepared by cg_init until scal->done.
 void run_fig1(stag_handle* h) {
+    if (h->resident && resident_fits(h->g, iterates_in_fp32(h))) {
+        run_fig1_resident(h);
+        return;
+    }
     const int K = h->opt.check_interval;
     const bool timing = h->opt.timing != 0;
     const bool graphs = h->opt.use_graphs != 0 && !timing;
@@ -356,6 +427,7 @@ void destroy_handle(stag_handle* h) {
     for (const stag_handle::Alloc& a : h->allocs) cudaFree(a.base);
     h->allocs.clear();
     if (h->scal_host) cudaFreeHost(h->scal_host);
+    if (h->timeout_host) cudaFreeHost(h->timeout_host);
     if (h->ev_in) cudaEventDestroy(h->ev_in);
     if (h->s) cudaStreamDestroy(h->s);
     delete h;
@@ -810,6 +882,19 @@ int stag_create_ex(stag_handle** out, const double* fat, const double* naik_long
         cuda_check(h, cudaMallocHost(reinterpret_cast<void**>(&h->scal_host), sizeof(CgScalars)),
                    "allocate pinned CG state");
         std::memset(h->scal_host, 0, sizeof(CgScalars));
+        h->resident = resident_fits(g, false) || (h->opt.inner != STAG_INNER_NONE && resident_fits(g, true));
+        if (h->resident) {
+            h->rwork.slots = dev_alloc<double>(h, sizeof(double) * 2 * kResidentMaxBlocks, "allocate exchange");
+            h->rwork.count = dev_alloc<unsigned int>(h, sizeof(unsigned int), "allocate exchange");
+            h->rwork.base = dev_alloc<unsigned int>(h, sizeof(unsigned int), "allocate exchange");
+            h->rwork.ns = dev_alloc<unsigned long long>(h, sizeof(unsigned long long) * STAG_KERNEL_COUNT,
+                                                        "allocate times");
+            cuda_check(h, cudaHostAlloc(reinterpret_cast<void**>(&h->timeout_host), sizeof(int), cudaHostAllocMapped),
+                       "allocate mapped flag");
+            *h->timeout_host = 0;
+            cuda_check(h, cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->rwork.timeout), h->timeout_host, 0),
+                       "map flag");
+        }
 
         const bool r12 = h->opt.link_recon == 12;
         pack_field(h, fat, h->fat64, h->fatff, r12 ? nullptr : h->fat32, h->fat16, h->fatb16, r12 ? h->fat32 : nullptr);

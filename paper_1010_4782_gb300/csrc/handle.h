@@ -11,6 +11,7 @@
 
 #include "../../include/stag.h"
 #include "stag_internal.cuh"
+#include "stag_kernels.h"
 
 namespace stag {
 struct KernelStat {
@@ -59,6 +60,10 @@ struct stag_handle {
     double* partials = nullptr;
     stag::CgScalars* scal = nullptr;
     stag::CgScalars* scal_host = nullptr;  // pinned
+    // small lattices: the iterations in one launch (resident.cu)
+    bool resident = false;
+    stag::ResidentWork rwork{nullptr, nullptr, nullptr, nullptr, nullptr};
+    int* timeout_host = nullptr;  // host-mapped: a bounded device-side wait ran out
     // graphs
     cudaGraphExec_t graph = nullptr;
     // timing

@@ -91,6 +91,36 @@ void launch_dslash_b16(const Geom& g, int out_parity, const __nv_bfloat162* fat,
                        const __nv_bfloat162* in, __nv_bfloat162* out, Epilogue epi, const __nv_bfloat162* src,
                        double m2, CgScalars* scal, double* partials, cudaStream_t s);
 
+// ---- the iterations of Fig. 1 in one cooperative launch, small lattices (resident.cu)
+constexpr int kResidentMaxBlocks = 256;
+struct ResidentWork {
+    double* slots;           // [2][kResidentMaxBlocks]: the blocks' partial sums
+    unsigned int* count;     // arrivals so far, zero at first
+    unsigned int* base;      // their number when the last launch ended, zero at first
+    int* timeout;            // host-mapped, set to 1 when a bounded wait ran out
+    unsigned long long* ns;  // nullable: time of D_oe, D_eo, the x/r update and the d update, added up
+};
+// Does every site get a thread of its own at once?  (fp32: FP32 arithmetic)
+bool resident_fits(const Geom& g, bool fp32);
+// At most `iters` iterations from the state in scal (returns at once if it is done);
+// at the end r, d and x are the iterate's, as after the kernels of blas.cu.
+cudaError_t launch_resident_f64(const Geom& g, const LinkSet& L, double2* d, double2* t, double2* r, double2* x,
+                                CgScalars* scal, const ResidentWork& w, int iters, cudaStream_t s);
+// fold: iterations between additions of the float-float increment to x (also at the end)
+cudaError_t launch_resident_ff(const Geom& g, const LinkSet& L, float4* d, float4* t, float4* r, double2* x,
+                               CgScalars* scal, const ResidentWork& w, int iters, int fold, cudaStream_t s);
+// The low-precision links of a handle: one of the storage types
+struct LoLinks {
+    const float2 *fat32 = nullptr, *lng32 = nullptr;
+    const __half2 *fat16 = nullptr, *lng16 = nullptr;
+    const __nv_bfloat162 *fatb16 = nullptr, *lngb16 = nullptr;
+    bool two_row_fat = false;    // fat32 holds two rows per link (12-parameter form)
+    bool vectors32 = false;      // FP16 links with FP32 vectors
+    float lng_inv_scale = 0.f;   // two-row FP32 Naik links: 1 / scale
+};
+cudaError_t launch_resident_lo(const Geom& g, const LoLinks& L, void* d, void* t, void* r, float2* y, CgScalars* scal,
+                               const ResidentWork& w, int iters, cudaStream_t s);
+
 // ---- CG vector kernels and reductions (blas.cu)
 // kBlock-thread blocks that fill every SM of the current device once (grid of
 // the grid-stride update kernels, whose grid reduction then has few partials)
