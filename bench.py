@@ -128,8 +128,8 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-DSLASH_SOURCES = ("dslash.cu", "dirac.cuh", "ff.cuh", "stag_internal.cuh")
-MULTI_SOURCES = ("multi.cu", "multi.cuh", "stag_internal.cuh")
+DSLASH_SOURCES = ("dslash.cu", "dirac.cuh", "links.cuh", "ff.cuh", "stag_internal.cuh")
+MULTI_SOURCES = ("multi.cu", "multi.cuh", "links.cuh", "stag_internal.cuh")
 
 
 def dslash_source_hash(files=DSLASH_SOURCES):

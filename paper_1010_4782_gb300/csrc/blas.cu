@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kBlock) cg_update_xr_ff_kernel(Geom g, float4*
         }
     }
     double total;
-    if (grid_sum_last_block<kBlock>(ff_acc_to_double(n2), partials, &scal->counter, &total)) {
+    if (grid_sum_last_block<kBlock>(n2, partials, &scal->counter, &total)) {
         if (threadIdx.x == 0) finish_delta(scal, total);
     }
 }

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kBlock) lo_update_xr_kernel(Geom g, float2* __
         }
     }
     double total;
-    if (grid_sum_last_block<kBlock>((double)acc, partials, &scal->counter, &total)) {
+    if (grid_sum_last_block<kBlock>(FFAcc{acc, 0.f}, partials, &scal->counter, &total)) {
         if (threadIdx.x == 0) {
             CgScalars* sc = scal;
             sc->delta_old = sc->delta_new;

@@ -9,6 +9,7 @@
 #include <type_traits>
 
 #include "ff.cuh"
+#include "links.cuh"
 #include "stag_kernels.h"
 
 namespace stag {
@@ -24,10 +25,14 @@ struct ArithF64 {
     static __device__ __forceinline__ C ldl(const TL* p) { return ld(p); }
     struct Acc {
         double2 c[3];
+        double dot;
     };
+    using Sum = double;  // of a dot product
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return a.dot; }
     static __device__ __forceinline__ void zero(Acc& a) {
 #pragma unroll
         for (int r = 0; r < 3; ++r) a.c[r] = make_double2(0.0, 0.0);
+        a.dot = 0.0;
     }
     // a_r += sum_c u_c v_c
     static __device__ __forceinline__ void row_fwd(Acc& a, int r, C u0, C u1, C u2, C v0, C v1, C v2) {
@@ -42,12 +47,12 @@ struct ArithF64 {
         cmsc_conj(a.c[r], u2, v2);
     }
     static __device__ __forceinline__ T store_val(const Acc& a, int r) { return a.c[r]; }
-    // o = m2 * s - acc_r; dot += Re(conj(s) o)
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2, double& dot) {
+    // o = m2 * s - acc_r; the dot product += Re(conj(s) o)
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2) {
         const double2 d = a.c[r];
         const double2 o = make_double2(fma(m2, s.x, -d.x), fma(m2, s.y, -d.y));
-        dot = fma(s.x, o.x, dot);
-        dot = fma(s.y, o.y, dot);
+        a.dot = fma(s.x, o.x, a.dot);
+        a.dot = fma(s.y, o.y, a.dot);
         return o;
     }
 };
@@ -78,14 +83,14 @@ struct ArithFF {
     static __device__ __forceinline__ T store_val(const Acc& a, int r) {
         return ff_cplx(ff_result(a.re[r]), ff_result(a.im[r]));
     }
-    // o = m2 * s - acc_r in float-float; Re(conj(s) o) accumulated in float-float,
-    // converted to FP64 once per thread (dot is only valid after the last row).
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double, float2 m2, double& dot) {
+    using Sum = FFAcc;
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return a.dot; }
+    // o = m2 * s - acc_r in float-float; Re(conj(s) o) accumulated in float-float
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double, float2 m2) {
         const float2 re = ff_fma(m2, ff_re(s), ff_neg(ff_result(a.re[r])));
         const float2 im = ff_fma(m2, ff_im(s), ff_neg(ff_result(a.im[r])));
         const float4 o = ff_cplx(re, im);
         ff_redot_acc(a.dot, s, o);
-        if (r == 2) dot = ff_acc_to_double(a.dot);
         return o;
     }
 };
@@ -119,12 +124,13 @@ struct ArithF32 {
         cmscf_conj(a.c[r], u2, v2);
     }
     static __device__ __forceinline__ T store_val(const Acc& a, int r) { return a.c[r]; }
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double, float2 m2, double& dot) {
+    using Sum = FFAcc;
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return FFAcc{a.dot, 0.f}; }
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double, float2 m2) {
         const float2 d = a.c[r];
         const float2 o = make_float2(fmaf(m2.x, s.x, -d.x), fmaf(m2.x, s.y, -d.y));
         a.dot = fmaf(s.x, o.x, a.dot);
         a.dot = fmaf(s.y, o.y, a.dot);
-        if (r == 2) dot = (double)a.dot;
         return o;
     }
 };
@@ -139,6 +145,8 @@ struct ArithH16 {
     static constexpr bool kRecon = false;
     static __device__ __forceinline__ C ldl(const TL* p) { return ld(p); }
     using Acc = ArithF32::Acc;
+    using Sum = ArithF32::Sum;
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
     static __device__ __forceinline__ void zero(Acc& a) { ArithF32::zero(a); }
     static __device__ __forceinline__ void row_fwd(Acc& a, int r, C u0, C u1, C u2, C v0, C v1, C v2) {
         ArithF32::row_fwd(a, r, u0, u1, u2, v0, v1, v2);
@@ -147,8 +155,8 @@ struct ArithH16 {
         ArithF32::row_bwd(a, r, u0, u1, u2, v0, v1, v2);
     }
     static __device__ __forceinline__ T store_val(const Acc& a, int r) { return __float22half2_rn(a.c[r]); }
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f, double& dot) {
-        return __float22half2_rn(ArithF32::epilogue(a, r, s, m2, m2f, dot));
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f) {
+        return __float22half2_rn(ArithF32::epilogue(a, r, s, m2, m2f));
     }
 };
 
@@ -163,6 +171,8 @@ struct ArithB16 {
     static constexpr bool kRecon = false;
     static __device__ __forceinline__ C ldl(const TL* p) { return ld(p); }
     using Acc = ArithF32::Acc;
+    using Sum = ArithF32::Sum;
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
     static __device__ __forceinline__ void zero(Acc& a) { ArithF32::zero(a); }
     static __device__ __forceinline__ void row_fwd(Acc& a, int r, C u0, C u1, C u2, C v0, C v1, C v2) {
         ArithF32::row_fwd(a, r, u0, u1, u2, v0, v1, v2);
@@ -171,8 +181,8 @@ struct ArithB16 {
         ArithF32::row_bwd(a, r, u0, u1, u2, v0, v1, v2);
     }
     static __device__ __forceinline__ T store_val(const Acc& a, int r) { return __float22bfloat162_rn(a.c[r]); }
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f, double& dot) {
-        return __float22bfloat162_rn(ArithF32::epilogue(a, r, s, m2, m2f, dot));
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f) {
+        return __float22bfloat162_rn(ArithF32::epilogue(a, r, s, m2, m2f));
     }
 };
 
@@ -189,6 +199,8 @@ struct ArithF32R {
     static __device__ __forceinline__ C ld(const T* p) { return __ldg(p); }
     static __device__ __forceinline__ C ldl(const TL* p) { return __ldg(p); }
     using Acc = ArithF32::Acc;
+    using Sum = ArithF32::Sum;
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
     static __device__ __forceinline__ void zero(Acc& a) { ArithF32::zero(a); }
     static __device__ __forceinline__ void row_fwd(Acc& a, int r, C u0, C u1, C u2, C v0, C v1, C v2) {
         ArithF32::row_fwd(a, r, u0, u1, u2, v0, v1, v2);
@@ -197,8 +209,8 @@ struct ArithF32R {
         ArithF32::row_bwd(a, r, u0, u1, u2, v0, v1, v2);
     }
     static __device__ __forceinline__ T store_val(const Acc& a, int r) { return ArithF32::store_val(a, r); }
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f, double& dot) {
-        return ArithF32::epilogue(a, r, s, m2, m2f, dot);
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f) {
+        return ArithF32::epilogue(a, r, s, m2, m2f);
     }
 };
 
@@ -213,6 +225,8 @@ struct ArithL16 {
     static __device__ __forceinline__ C ld(const T* p) { return __ldg(p); }
     static __device__ __forceinline__ C ldl(const TL* p) { return __half22float2(__ldg(p)); }
     using Acc = ArithF32::Acc;
+    using Sum = ArithF32::Sum;
+    static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
     static __device__ __forceinline__ void zero(Acc& a) { ArithF32::zero(a); }
     static __device__ __forceinline__ void row_fwd(Acc& a, int r, C u0, C u1, C u2, C v0, C v1, C v2) {
         ArithF32::row_fwd(a, r, u0, u1, u2, v0, v1, v2);
@@ -221,8 +235,8 @@ struct ArithL16 {
         ArithF32::row_bwd(a, r, u0, u1, u2, v0, v1, v2);
     }
     static __device__ __forceinline__ T store_val(const Acc& a, int r) { return ArithF32::store_val(a, r); }
-    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f, double& dot) {
-        return ArithF32::epilogue(a, r, s, m2, m2f, dot);
+    static __device__ __forceinline__ T epilogue(Acc& a, int r, C s, double m2, float2 m2f) {
+        return ArithF32::epilogue(a, r, s, m2, m2f);
     }
 };
 
@@ -230,8 +244,8 @@ template <class A>
 struct DslashParams {
     Geom g;
     int P;                     // output parity
-    const typename A::TL* fat;  // [2][4][9][vs]
-    const typename A::TL* lng;  // [2][4][9][vs] or nullptr
+    const typename A::TL* fat;  // [2][4][9][vs], or the words of links.cuh
+    const typename A::TL* lng;  // the same, or nullptr
     const typename A::T* in;   // [3][vs], parity 1-P
     typename A::T* out;        // [3][vs], parity P
     const typename A::T* src;  // [3][vs], parity P (EPI_AXPY / EPI_CG)
@@ -241,6 +255,7 @@ struct DslashParams {
     double* partials;
     int i0, i1;                // output sites [i0, i1) of parity P
     float2 lng_s = make_float2(0.f, 0.f);  // NAIK == 2: 1 / scale of the two-row Naik links (float-float)
+    int epi = EPI_PLAIN;       // the epilogue of a kernel that takes it at run time
 };
 
 // Link entries 6..8 (the third row) from the first two: eta * conj(row0 x row1).
@@ -250,11 +265,8 @@ __device__ __forceinline__ float2 cross_conj(float2 a1, float2 b2, float2 a2, fl
     const float im = a1.x * b2.y + a1.y * b2.x - (a2.x * b1.y + a2.y * b1.x);
     return make_float2(eta * re, -eta * im);
 }
-template <class A>
-__device__ __forceinline__ void load_recon(typename A::C (&U)[9], const typename A::TL* __restrict__ u, size_t vs,
-                                           float eta) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) U[k] = A::ldl(u + k * vs);
+__device__ __forceinline__ void load_recon(float2 (&U)[9], const float2* __restrict__ u, size_t vs, int i, float eta) {
+    load_link<6>(U, u, vs, i);
     U[6] = cross_conj(U[1], U[5], U[2], U[4], eta);
     U[7] = cross_conj(U[2], U[3], U[0], U[5], eta);
     U[8] = cross_conj(U[0], U[4], U[1], U[3], eta);
@@ -287,16 +299,23 @@ __device__ __forceinline__ void hop_bwd_ffr(ArithFF::Acc& acc, const float4* __r
     for (int r = 0; r < 3; ++r) ArithFF::row_bwd(acc, r, U[r], U[3 + r], U[6 + r], v0, v1, v2);
 }
 
+// acc += U in(nb) with site i's link of part u (its [parity][mu]); backward: acc -= U^dag in(nb).
+// FP32 arithmetic takes the whole link in 16-byte words; FP64 and float-float, whose
+// entries are words, a row (or column) at a time, which needs fewer registers at once.
 template <class A>
-__device__ __forceinline__ void hop_fwd(typename A::Acc& acc, const typename A::TL* __restrict__ u,
+__device__ __forceinline__ void hop_fwd(typename A::Acc& acc, const typename A::TL* __restrict__ u, int i,
                                         const typename A::T* __restrict__ in, int nb, size_t vs, float eta = 1.f) {
     const typename A::C v0 = A::ld(in + nb), v1 = A::ld(in + vs + nb), v2 = A::ld(in + 2 * vs + nb);
-    if constexpr (A::kRecon) {
-        typename A::C U[9];
-        load_recon<A>(U, u, vs, eta);
+    if constexpr (std::is_same<typename A::C, float2>::value) {
+        float2 U[9];
+        if constexpr (A::kRecon)
+            load_recon(U, u, vs, i, eta);
+        else
+            load_link<9>(U, u, vs, i);
 #pragma unroll
         for (int r = 0; r < 3; ++r) A::row_fwd(acc, r, U[3 * r], U[3 * r + 1], U[3 * r + 2], v0, v1, v2);
     } else {
+        u += i;
 #pragma unroll
         for (int r = 0; r < 3; ++r)
             A::row_fwd(acc, r, A::ldl(u + (3 * r) * vs), A::ldl(u + (3 * r + 1) * vs), A::ldl(u + (3 * r + 2) * vs),
@@ -305,16 +324,20 @@ __device__ __forceinline__ void hop_fwd(typename A::Acc& acc, const typename A::
 }
 
 template <class A>
-__device__ __forceinline__ void hop_bwd(typename A::Acc& acc, const typename A::TL* __restrict__ u,
-                                        const typename A::T* __restrict__ in, int nb, size_t vs, float eta = 1.f) {
-    const typename A::C v0 = A::ld(in + nb), v1 = A::ld(in + vs + nb), v2 = A::ld(in + 2 * vs + nb);
-    // (U^dag v)_r = sum_c conj(U_cr) v_c
-    if constexpr (A::kRecon) {
-        typename A::C U[9];
-        load_recon<A>(U, u, vs, eta);
+__device__ __forceinline__ void hop_bwd(typename A::Acc& acc, const typename A::TL* __restrict__ u, int i,
+                                        const typename A::T* __restrict__ in, size_t vs, float eta = 1.f) {
+    const typename A::C v0 = A::ld(in + i), v1 = A::ld(in + vs + i), v2 = A::ld(in + 2 * vs + i);
+    // (U^dag v)_r = sum_c conj(U_cr) v_c; the link is the neighbour's own
+    if constexpr (std::is_same<typename A::C, float2>::value) {
+        float2 U[9];
+        if constexpr (A::kRecon)
+            load_recon(U, u, vs, i, eta);
+        else
+            load_link<9>(U, u, vs, i);
 #pragma unroll
         for (int r = 0; r < 3; ++r) A::row_bwd(acc, r, U[r], U[3 + r], U[6 + r], v0, v1, v2);
     } else {
+        u += i;
 #pragma unroll
         for (int r = 0; r < 3; ++r)
             A::row_bwd(acc, r, A::ldl(u + r * vs), A::ldl(u + (3 + r) * vs), A::ldl(u + (6 + r) * vs), v0, v1, v2);
@@ -351,14 +374,14 @@ __device__ __forceinline__ void dslash_site(const DslashParams<A>& p, int i, typ
             // eta_mu(x) = eta_mu(x - mu): the phase of both links of this direction
             const int ps = (mu >= 1 ? x : 0) + (mu >= 2 ? y : 0) + (mu >= 3 ? z : 0);
             const float eta = (ps & 1) ? -1.f : 1.f;
-            hop_fwd<A>(acc, p.fat + ((size_t)(P * 4 + mu) * A::kEntries) * vs + i, p.in, f1, vs, eta);
-            hop_bwd<A>(acc, p.fat + ((size_t)(Q * 4 + mu) * A::kEntries) * vs + b1, p.in, b1, vs, eta);
+            hop_fwd<A>(acc, p.fat + ((size_t)(P * 4 + mu) * A::kEntries) * vs, i, p.in, f1, vs, eta);
+            hop_bwd<A>(acc, p.fat + ((size_t)(Q * 4 + mu) * A::kEntries) * vs, b1, p.in, vs, eta);
             if constexpr (NAIK == 1) {
                 const int h = g.hop3[mu];
                 const int f3 = neighbour(g, x, y, z, t, mu, h, true);
                 const int b3 = neighbour(g, x, y, z, t, mu, h, false);
-                hop_fwd<A>(acc, p.lng + ((size_t)(P * 4 + mu) * 9) * vs + i, p.in, f3, vs);
-                hop_bwd<A>(acc, p.lng + ((size_t)(Q * 4 + mu) * 9) * vs + b3, p.in, b3, vs);
+                hop_fwd<A>(acc, p.lng + ((size_t)(P * 4 + mu) * 9) * vs, i, p.in, f3, vs);
+                hop_bwd<A>(acc, p.lng + ((size_t)(Q * 4 + mu) * 9) * vs, b3, p.in, vs);
             }
         }
         if constexpr (NAIK == 2) {
@@ -379,8 +402,8 @@ __device__ __forceinline__ void dslash_site(const DslashParams<A>& p, int i, typ
                     // FP32 (the mixed-precision iteration): the same rows, the third
                     // rebuilt in FP32 with the factor eta / scale
                     const float s = (ps & 1) ? -p.lng_s.x : p.lng_s.x;
-                    hop_fwd<ArithF32R>(acc, p.lng + ((size_t)(P * 4 + mu) * 6) * vs + i, p.in, f3, vs, s);
-                    hop_bwd<ArithF32R>(acc, p.lng + ((size_t)(Q * 4 + mu) * 6) * vs + b3, p.in, b3, vs, s);
+                    hop_fwd<ArithF32R>(acc, p.lng + ((size_t)(P * 4 + mu) * 6) * vs, i, p.in, f3, vs, s);
+                    hop_bwd<ArithF32R>(acc, p.lng + ((size_t)(Q * 4 + mu) * 6) * vs, b3, p.in, vs, s);
                 }
             }
         }

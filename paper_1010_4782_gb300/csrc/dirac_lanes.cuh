@@ -46,19 +46,20 @@ __device__ __forceinline__ void swap_if(float4& a, float4& b, bool sw) {
 // part's sign).  The transpose is taken by the order of the loads, or for
 // two-row links by exchanging entries after the third row is rebuilt.
 template <class A, int ENTRIES>
-__device__ __forceinline__ void lane_hop(typename A::Acc& acc, const typename A::TL* __restrict__ u,
+__device__ __forceinline__ void lane_hop(typename A::Acc& acc, const typename A::TL* __restrict__ u, int li,
                                          const typename A::T* in, int nb, size_t vs, bool bwd, float2 s) {
     using C = typename A::C;
     C U[9], v[3];
-    if constexpr (ENTRIES == 9) {
+    constexpr bool kWords = std::is_same<C, float2>::value;  // links in 16-byte words of several entries
+    if constexpr (ENTRIES == 9 && !kWords) {
         const size_t sr = (bwd ? 1 : 3) * vs, sc = (bwd ? 3 : 1) * vs;
+        u += li;
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
             for (int c = 0; c < 3; ++c) U[3 * r + c] = A::ldl(u + r * sr + c * sc);
     } else {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) U[k] = A::ldl(u + k * vs);
+        load_link<ENTRIES>(U, u, vs, li);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) v[c] = conj_if(ld_vec(in + c * vs + nb), bwd);
@@ -72,6 +73,8 @@ __device__ __forceinline__ void lane_hop(typename A::Acc& acc, const typename A:
             U[7] = cross_conj(U[2], U[3], U[0], U[5], s.x);
             U[8] = cross_conj(U[0], U[4], U[1], U[3], s.x);
         }
+    }
+    if constexpr (ENTRIES == 6 || kWords) {
         swap_if(U[1], U[3], bwd);
         swap_if(U[2], U[6], bwd);
         swap_if(U[5], U[7], bwd);
@@ -143,11 +146,11 @@ __device__ __forceinline__ void lane_directions(const LaneField<A>& f, int P, co
         };
         const bool odd = ((mu >= 1 ? x : 0) + (mu >= 2 ? y : 0) + (mu >= 3 ? z : 0)) & 1;
         const int n1 = nbr(1);
-        lane_hop<A, EF>(acc, f.fat + (size_t)((plane + mu) * EF) * vs + (bwd ? n1 : i), in, n1, vs, bwd,
+        lane_hop<A, EF>(acc, f.fat + (size_t)((plane + mu) * EF) * vs, bwd ? n1 : i, in, n1, vs, bwd,
                         make_float2(odd ? -1.f : 1.f, 0.f));
         if constexpr (NAIK != 0) {
             const int n3 = nbr(mu == 0 ? g.hop3[0] : mu == 1 ? g.hop3[1] : mu == 2 ? g.hop3[2] : g.hop3[3]);
-            lane_hop<AL, EL>(acc, f.lng + (size_t)((plane + mu) * EL) * vs + (bwd ? n3 : i), in, n3, vs, bwd,
+            lane_hop<AL, EL>(acc, f.lng + (size_t)((plane + mu) * EL) * vs, bwd ? n3 : i, in, n3, vs, bwd,
                              odd ? make_float2(-f.lng_s.x, -f.lng_s.y) : f.lng_s);
         }
     }

@@ -41,11 +41,18 @@ constexpr int dslash_min_blocks() {
     return std::is_same<A, ArithFF>::value ? 2 : (NAIK == 2 ? 3 : 4);
 }
 
+// The float-float kernels take their epilogue at run time (EPI = kEpiRuntime): their
+// unrolled stencil is some 200 KB of code, and D_oe and D_eo as two kernels refilled the
+// instruction cache at every launch (28^3 x 96: 386 and 411 us when one is repeated, 828
+// us in turn, as one kernel 801 us; 24^3 x 48: 132, 147 and 311 us, as one kernel 278 us).
+constexpr int kEpiRuntime = -1;
+
 template <class A, int NAIK, int EPI>
 __global__ void __launch_bounds__(kBlock, dslash_min_blocks<A, NAIK>()) dslash_kernel(const DslashParams<A> p) {
     // Inside a solver iteration (CG state given): return once the loop has
     // stopped, so that the rest of a captured block of iterations costs nothing.
     if (p.scal && p.scal->done) return;
+    const int epi = EPI == kEpiRuntime ? p.epi : EPI;
     const Geom& g = p.g;
     const int i = p.i0 + blockIdx.x * kBlock + threadIdx.x;
     const size_t vs = (size_t)g.vs;
@@ -58,16 +65,16 @@ __global__ void __launch_bounds__(kBlock, dslash_min_blocks<A, NAIK>()) dslash_k
     SrcT srcv[3];
     double m2 = 0.0;
     float2 m2_ff = make_float2(0.f, 0.f);
-    if (EPI != EPI_PLAIN) {
-        m2 = (EPI == EPI_CG) ? p.scal->m2 : p.m2;
-        m2_ff = (EPI == EPI_CG) ? p.scal->m2_ff : p.m2_ff;
+    if (epi != EPI_PLAIN) {
+        m2 = (epi == EPI_CG) ? p.scal->m2 : p.m2;
+        m2_ff = (epi == EPI_CG) ? p.scal->m2_ff : p.m2_ff;
         if (active) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) srcv[r] = A::ld(p.src + r * vs + i);
         }
     }
     if (active) dslash_site<A, NAIK>(p, i, acc);
-    if (EPI == EPI_PLAIN) {
+    if (epi == EPI_PLAIN) {
         if (active) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) p.out[r * vs + i] = A::store_val(acc, r);
@@ -75,14 +82,13 @@ __global__ void __launch_bounds__(kBlock, dslash_min_blocks<A, NAIK>()) dslash_k
         return;
     }
     // out = m2 * src - D in
-    double dot = 0.0;
     if (active) {
 #pragma unroll
-        for (int r = 0; r < 3; ++r) p.out[r * vs + i] = A::epilogue(acc, r, srcv[r], m2, m2_ff, dot);
+        for (int r = 0; r < 3; ++r) p.out[r * vs + i] = A::epilogue(acc, r, srcv[r], m2, m2_ff);
     }
-    if (EPI == EPI_CG) {
+    if (epi == EPI_CG) {
         double total;
-        if (grid_sum_last_block<kBlock>(dot, p.partials, &p.scal->counter, &total)) {
+        if (grid_sum_last_block<kBlock>(A::dot(acc), p.partials, &p.scal->counter, &total)) {
             if (threadIdx.x == 0) {
                 CgScalars* sc = p.scal;
                 sc->pAp = total;
@@ -141,13 +147,12 @@ __global__ void __launch_bounds__(kBlock, 3) dslash_list_kernel(const SysDirac* 
         else
             dslash_site<A, 0>(p, i, acc);
         const size_t vs = (size_t)sd.g.vs;
-        double dot = 0.0;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             if (EPI == EPI_PLAIN)
                 p.out[r * vs + i] = A::store_val(acc, r);
             else
-                p.out[r * vs + i] = A::epilogue(acc, r, A::ld(p.src + r * vs + i), p.m2, p.m2_ff, dot);
+                p.out[r * vs + i] = A::epilogue(acc, r, A::ld(p.src + r * vs + i), p.m2, p.m2_ff);
         }
     }
 }
@@ -183,11 +188,16 @@ static void launch_one(const DslashParams<A>& p, int naik, cudaStream_t s) {
 }
 
 template <class A>
-static void launch_any(const DslashParams<A>& p, int naik, Epilogue epi, cudaStream_t s) {
-    switch (epi) {
-        case EPI_PLAIN: launch_one<A, EPI_PLAIN>(p, naik, s); break;
-        case EPI_AXPY: launch_one<A, EPI_AXPY>(p, naik, s); break;
-        default: launch_one<A, EPI_CG>(p, naik, s); break;
+static void launch_any(DslashParams<A> p, int naik, Epilogue epi, cudaStream_t s) {
+    if constexpr (std::is_same<A, ArithFF>::value) {
+        p.epi = epi;
+        launch_one<A, kEpiRuntime>(p, naik, s);
+    } else {
+        switch (epi) {
+            case EPI_PLAIN: launch_one<A, EPI_PLAIN>(p, naik, s); break;
+            case EPI_AXPY: launch_one<A, EPI_AXPY>(p, naik, s); break;
+            default: launch_one<A, EPI_CG>(p, naik, s); break;
+        }
     }
 }
 

@@ -15,7 +15,10 @@
 // and the last block of each group sums them in block order.
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "ff.cuh"
+#include "links.cuh"
 #include "multi.cuh"
 
 namespace stag {
@@ -215,16 +218,15 @@ __device__ __forceinline__ void store_rb(float2* p, const float2 (&v)[RB]) {
     }
 }
 
-// acc[r][j] += U v (fwd, U at the output site) or -= U^dag v (bwd, U at the neighbour)
-template <int RB, bool BWD>
+// acc[r][j] += U v (fwd, U at the output site) or -= U^dag v (bwd, U at the neighbour).
+// The links are read once: Ld = LoadStreaming loads them evict-first, so that they do not
+// push the reused input vectors out of L2.
+template <int RB, bool BWD, class Ld>
 __device__ __forceinline__ void multi_hop(float2 (&acc)[3][RB], const float2* __restrict__ u,
-                                          const float2* __restrict__ in, int nb, size_t vs, int rpad, int roff,
-                                          bool stream_links = false) {
+                                          int li, const float2* __restrict__ in, int nb, size_t vs, int rpad,
+                                          int roff) {
     float2 U[9];
-    // the links are read once: with stream_links they are loaded as streaming
-    // (evict-first) data, so that they do not push the reused input vectors out of L2
-#pragma unroll
-    for (int k = 0; k < 9; ++k) U[k] = stream_links ? __ldcs(u + k * vs) : __ldg(u + k * vs);
+    load_link<9, Ld>(U, u, vs, li);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         float2 v[RB];
@@ -267,6 +269,7 @@ __global__ void __launch_bounds__(BS, (RB == 8 ? 512 / BS : 1)) multi_dslash_ker
 #pragma unroll
     for (int j = 0; j < RB; ++j) dotf[j] = 0.f;
     constexpr bool kSweep = MODE != 0;
+    using Ld = typename std::conditional<kSweep, LoadStreaming, LoadCached>::type;
     const int tile0 = kSweep ? blk : tile_end(blk - 1, ntiles, nblk);
     const int tile1 = kSweep ? ntiles : tile_end(blk, ntiles, nblk);
     const int step = kSweep ? nblk : 1;
@@ -284,18 +287,14 @@ __global__ void __launch_bounds__(BS, (RB == 8 ? 512 / BS : 1)) multi_dslash_ker
         for (int mu = 0; mu < 4; ++mu) {
             const int f1 = nbr_index(g, x, y, z, t, mu, 1, true);
             const int b1 = nbr_index(g, x, y, z, t, mu, 1, false);
-            multi_hop<RB, false>(acc, G.fat + ((size_t)(P * 4 + mu) * 9) * vs + i, in, f1, vs, G.rpad, l.roff,
-                                 kSweep);
-            multi_hop<RB, true>(acc, G.fat + ((size_t)(Q * 4 + mu) * 9) * vs + b1, in, b1, vs, G.rpad, l.roff,
-                                kSweep);
+            multi_hop<RB, false, Ld>(acc, G.fat + ((size_t)(P * 4 + mu) * 9) * vs, i, in, f1, vs, G.rpad, l.roff);
+            multi_hop<RB, true, Ld>(acc, G.fat + ((size_t)(Q * 4 + mu) * 9) * vs, b1, in, b1, vs, G.rpad, l.roff);
             if (G.lng) {
                 const int h = g.hop3[mu];
                 const int f3 = nbr_index(g, x, y, z, t, mu, h, true);
                 const int b3 = nbr_index(g, x, y, z, t, mu, h, false);
-                multi_hop<RB, false>(acc, G.lng + ((size_t)(P * 4 + mu) * 9) * vs + i, in, f3, vs, G.rpad,
-                                     l.roff, kSweep);
-                multi_hop<RB, true>(acc, G.lng + ((size_t)(Q * 4 + mu) * 9) * vs + b3, in, b3, vs, G.rpad,
-                                    l.roff, kSweep);
+                multi_hop<RB, false, Ld>(acc, G.lng + ((size_t)(P * 4 + mu) * 9) * vs, i, in, f3, vs, G.rpad, l.roff);
+                multi_hop<RB, true, Ld>(acc, G.lng + ((size_t)(Q * 4 + mu) * 9) * vs, b3, in, b3, vs, G.rpad, l.roff);
             }
         }
 #pragma unroll

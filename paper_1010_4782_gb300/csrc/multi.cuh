@@ -9,7 +9,7 @@ namespace stag {
 // stored right-hand-side innermost: v[(colour * vs + site) * rpad + rhs].
 struct MultiGroup {
     Geom g;
-    const float2* fat;  // FP32 SoA links [2][4][9][vs], eta folded
+    const float2* fat;  // FP32 links [2][4] in the words of links.cuh, eta folded
     const float2* lng;  // or nullptr
     float2* d;          // search directions
     float2* t;          // odd-parity intermediate D_oe d

@@ -4,13 +4,15 @@
 // ABI <-> internal vector conversions.
 #include "stag_kernels.h"
 #include "ff.cuh"
+#include "links.cuh"
 
 namespace stag {
 
 // One thread per (site, direction), direction fastest, so that a warp reads
 // contiguous AoS links (the input may be host memory read over the host link).
 // Reads the 9 complex entries of U_mu(x) (144 contiguous bytes), multiplies by
-// eta_mu(x) and scatters them into the 9 planes of its parity.
+// eta_mu(x) and scatters them into the 9 planes of its parity (FP64, float-float) or the
+// 16-byte words of links.cuh (FP32, FP16, BF16).
 __global__ void __launch_bounds__(kBlock) pack_links_kernel(Geom g, const double2* __restrict__ aos,
                                                             double2* __restrict__ soa64,
                                                             float4* __restrict__ soaff,
@@ -37,17 +39,18 @@ __global__ void __launch_bounds__(kBlock) pack_links_kernel(Geom g, const double
     const double eta = (phase_sum & 1) ? -1.0 : 1.0;
     const double2* src = aos + ((size_t)lex * 4 + mu) * 9;
     const size_t vs = (size_t)g.vs;
-    const size_t base = ((size_t)(P * 4 + mu) * 9) * vs + cb;
+    const size_t base = ((size_t)(P * 4 + mu) * 9) * vs;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         double2 u = src[k];
         u.x *= eta;
         u.y *= eta;
-        soa64[base + k * vs] = u;
-        if (soaff) soaff[base + k * vs] = ff_from_complex(u);
-        if (soa32) soa32[base + k * vs] = make_float2((float)u.x, (float)u.y);
-        if (soa16) soa16[base + k * vs] = __floats2half2_rn((float)u.x, (float)u.y);
-        if (soab16) soab16[base + k * vs] = __floats2bfloat162_rn((float)u.x, (float)u.y);
+        soa64[base + k * vs + cb] = u;
+        if (soaff) soaff[base + k * vs + cb] = ff_from_complex(u);
+        const size_t w32 = base + link_offset<9, float2>(k, cb, vs), w16 = base + link_offset<9, __half2>(k, cb, vs);
+        if (soa32) soa32[w32] = make_float2((float)u.x, (float)u.y);
+        if (soa16) soa16[w16] = __floats2half2_rn((float)u.x, (float)u.y);
+        if (soab16) soab16[w16] = __floats2bfloat162_rn((float)u.x, (float)u.y);
     }
 }
 
@@ -59,7 +62,7 @@ void launch_pack_links(const Geom& g, const double* aos, double2* soa64, float4*
                                                 soaff, soa32, soa16, soab16);
 }
 
-// Links with the first two rows only ([parity][mu][6][vs], eta folded), in FP32
+// Links with the first two rows only ([parity][mu], six entries, eta folded), in FP32
 // and/or float-float: the third row of an SU(3) matrix (times a scale) is the
 // conjugate cross product of the first two (Sec. 3.3), rebuilt in the Dirac
 // kernel.  Direction fastest, as above.
@@ -86,12 +89,12 @@ __global__ void __launch_bounds__(kBlock) pack_links_rows2_kernel(Geom g, const 
     const double eta = (phase_sum & 1) ? -1.0 : 1.0;
     const double2* src = aos + ((size_t)lex * 4 + mu) * 9;
     const size_t vs = (size_t)g.vs;
-    const size_t base = ((size_t)(P * 4 + mu) * 6) * vs + cb;
+    const size_t base = ((size_t)(P * 4 + mu) * 6) * vs;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
         const double2 u = make_double2(eta * src[k].x, eta * src[k].y);
-        if (soa32r) soa32r[base + k * vs] = make_float2((float)u.x, (float)u.y);
-        if (soaffr) soaffr[base + k * vs] = ff_from_complex(u);
+        if (soa32r) soa32r[base + link_offset<6, float2>(k, cb, vs)] = make_float2((float)u.x, (float)u.y);
+        if (soaffr) soaffr[base + k * vs + cb] = ff_from_complex(u);
     }
 }
 

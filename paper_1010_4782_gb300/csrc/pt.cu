@@ -104,8 +104,7 @@ __global__ void __launch_bounds__(256, CIN * COUT >= 64 ? 2 : 3)
             const Hop hp = pt_hop(g, links, P, i, x, y, z, t, mu, d);
             Pn = hp.Pn;
             nb = hp.nb;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) U[k] = __ldg(hp.u + k * vs);
+            load_link<9>(U, hp.u, vs, hp.li);
         }
 #pragma unroll
         for (int ci = 0; ci < CIN; ++ci) {
@@ -184,8 +183,7 @@ __global__ void __launch_bounds__(256) pt_wgrad_kernel(Geom g, const float2* __r
             const Hop hp = pt_hop(g, links, P, i, x, y, z, t, mu, d);
             Pn = hp.Pn;
             nb = hp.nb;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) U[k] = __ldg(hp.u + k * vs);
+            load_link<9>(U, hp.u, vs, hp.li);
         }
         float2 gv[OC][3];
 #pragma unroll
@@ -490,10 +488,17 @@ __global__ void pt_scale_kernel(Geom g, float2* v, const float2* w, float s) {
     }
 }
 
+// Offset of the FP64 links' element n ([parity][mu][9][vs]) in the words of links.cuh.
+template <class T>
+__device__ __forceinline__ size_t word_offset(size_t n, size_t vs) {
+    const size_t part = n / (9 * vs), k = n % (9 * vs) / vs, i = n % vs;
+    return part * 9 * vs + link_offset<9, T>((int)k, i, vs);
+}
+
 // FP32 copy of the eta-folded FP64 links
-__global__ void pt_links_kernel(const double2* __restrict__ in, float2* __restrict__ out, size_t n) {
+__global__ void pt_links_kernel(const double2* __restrict__ in, float2* __restrict__ out, size_t n, size_t vs) {
     const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) out[k] = make_float2((float)in[k].x, (float)in[k].y);
+    if (k < n) out[word_offset<float2>(k, vs)] = make_float2((float)in[k].x, (float)in[k].y);
 }
 
 // largest |Re|, |Im| of the entries (as FP32 bits, atomically into *out; NaNs ignored)
@@ -507,9 +512,10 @@ __global__ void pt_absmax_kernel(const double2* __restrict__ in, size_t n, unsig
 }
 
 // FP16 copy of the links divided by s
-__global__ void pt_links16_kernel(const double2* __restrict__ in, __half2* __restrict__ out, size_t n, double inv_s) {
+__global__ void pt_links16_kernel(const double2* __restrict__ in, __half2* __restrict__ out, size_t n, size_t vs,
+                                  double inv_s) {
     const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) out[k] = __floats2half2_rn((float)(in[k].x * inv_s), (float)(in[k].y * inv_s));
+    if (k < n) out[word_offset<__half2>(k, vs)] = __floats2half2_rn((float)(in[k].x * inv_s), (float)(in[k].y * inv_s));
 }
 
 // ------------------------------------------------ collapsed inference form
@@ -960,10 +966,10 @@ int stag_ptnet_create(stag_ptnet** out, stag_handle* h, int32_t precision, uint6
         handle_begin(h);
         const size_t nl = (size_t)2 * 4 * 9 * n->g.vs;
         n->links = static_cast<float2*>(palloc(n, nl * sizeof(float2), "allocate links"));
-        pt_links_kernel<<<(int)((nl + 255) / 256), 256, 0, S(n)>>>(h->fat64, n->links, nl);
+        pt_links_kernel<<<(int)((nl + 255) / 256), 256, 0, S(n)>>>(h->fat64, n->links, nl, (size_t)n->g.vs);
         if (h->lng64) {
             n->lng = static_cast<float2*>(palloc(n, nl * sizeof(float2), "allocate links"));
-            pt_links_kernel<<<(int)((nl + 255) / 256), 256, 0, S(n)>>>(h->lng64, n->lng, nl);
+            pt_links_kernel<<<(int)((nl + 255) / 256), 256, 0, S(n)>>>(h->lng64, n->lng, nl, (size_t)n->g.vs);
         }
         const size_t fv = (size_t)3 * n->g.vs * sizeof(float2);
         n->va = static_cast<float2*>(palloc(n, fv, "allocate vectors"));
@@ -989,7 +995,7 @@ int stag_ptnet_create(stag_ptnet** out, stag_handle* h, int32_t precision, uint6
             std::memcpy(&amax, &bits, sizeof(amax));
             n->links16_scale = (amax > 0.f && std::isfinite(amax)) ? std::exp2f(std::round(std::log2(amax))) : 1.f;
             n->links16 = static_cast<__half2*>(palloc(n, nl * sizeof(__half2), "allocate links"));
-            pt_links16_kernel<<<(int)((nl + 255) / 256), 256, 0, S(n)>>>(h->fat64, n->links16, nl,
+            pt_links16_kernel<<<(int)((nl + 255) / 256), 256, 0, S(n)>>>(h->fat64, n->links16, nl, (size_t)n->g.vs,
                                                                           1.0 / n->links16_scale);
         }
         n->grad = static_cast<float2*>(palloc(n, nw * sizeof(float2), "allocate gradients"));

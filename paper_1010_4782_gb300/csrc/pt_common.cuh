@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "links.cuh"
 #include "stag_kernels.h"
 
 namespace stag {
@@ -92,8 +93,9 @@ __device__ __forceinline__ int pt_neighbour(const Geom& g, int x, int y, int z, 
 // stored as L (float2, or __half2 for the two-hop inference kernels).
 template <class L>
 struct HopT {
-    int Pn, nb;
-    const L* u;
+    int Pn, nb;  // source site
+    int li;      // site whose link it is
+    const L* u;  // the link's [parity][mu] part (links.cuh)
 };
 using Hop = HopT<float2>;
 
@@ -103,19 +105,11 @@ __device__ __forceinline__ HopT<L> pt_hop(const Geom& g, const L* links, int P, 
     HopT<L> h;
     h.Pn = 1 - P;
     const size_t vs = (size_t)g.vs;
-    if (d == 0) {
-        h.nb = pt_neighbour(g, x, y, z, t, mu, true);
-        h.u = links + ((size_t)(P * 4 + mu) * 9) * vs + i;
-    } else {
-        h.nb = pt_neighbour(g, x, y, z, t, mu, false);
-        h.u = links + ((size_t)((1 - P) * 4 + mu) * 9) * vs + h.nb;
-    }
+    h.nb = pt_neighbour(g, x, y, z, t, mu, d == 0);
+    h.li = d == 0 ? i : h.nb;
+    h.u = links + ((size_t)((d == 0 ? P : 1 - P) * 4 + mu) * 9) * vs;
     return h;
 }
-
-// one link entry in FP32
-__device__ __forceinline__ float2 ldu(const float2* p) { return __ldg(p); }
-__device__ __forceinline__ float2 ldu(const __half2* p) { return __half22float2(__ldg(p)); }
 
 // t = U v (d = 0) or U^dag v (d = 1), on packed FP32 pairs: per row the real
 // and the imaginary parts of the link each multiply the whole complex v[c],
@@ -163,8 +157,7 @@ __device__ __forceinline__ void pt_chi_site(const Geom& g, const L* __restrict__
         const int mu = (q - 1) >> 1, d = (q - 1) & 1;
         const HopT<L> hp = pt_hop(g, links, 1, i, x, y, z, t, mu, d);
         float2 U[9], v[3], tv[3];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) U[k] = ldu(hp.u + k * vs);
+        load_link<9>(U, hp.u, vs, hp.li);
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[c] = ldc(r + c * vs + hp.nb);
         pt_apply(U, d, v, tv);
@@ -199,8 +192,7 @@ __device__ __forceinline__ void pt_out_site(const Geom& g, const L* __restrict__
         const int mu = (p - 1) >> 1, d = (p - 1) & 1;
         const HopT<L> hp = pt_hop(g, links, 0, i, x, y, z, t, mu, d);
         float2 U[9], v[3], tv[3];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) U[k] = ldu(hp.u + k * vs);
+        load_link<9>(U, hp.u, vs, hp.li);
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[c] = ldc(chi + ((size_t)(p - 1) * 3 + c) * vs + hp.nb);
         pt_apply(U, d, v, tv);

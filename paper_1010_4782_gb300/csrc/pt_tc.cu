@@ -212,8 +212,7 @@ __global__ void __launch_bounds__(kTileRows) pt_mix8_tc_kernel(Geom g, const flo
                 const Hop hp = pt_hop(g, links, P, i, x, y, z, t, mu, d);
                 Pn = hp.Pn;
                 nb = hp.nb;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) U[k] = __ldg(hp.u + k * vs);
+                load_link<9>(U, hp.u, vs, hp.li);
             }
             uint8_t* row = rowA + b * kABuf;
 #pragma unroll
@@ -362,8 +361,7 @@ __global__ void __launch_bounds__(256) pt_transport_sum_kernel(Geom g, const flo
         const int mu = (p - 1) >> 1, d = (p - 1) & 1;
         const Hop hp = pt_hop(g, links, 0, i, x, y, z, t, mu, d);
         float2 U[9], v[3], tv[3];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) U[k] = __ldg(hp.u + k * vs);
+        load_link<9>(U, hp.u, vs, hp.li);
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[c] = ldc(phi + fidx(p - 1, c, hp.Pn, hp.nb, vs, kHidden));
         pt_apply(U, d, v, tv);

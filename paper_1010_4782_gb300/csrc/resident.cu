@@ -63,16 +63,7 @@ __device__ __forceinline__ unsigned long long now_ns() {
 // -------------------------------------------- the vector steps, per arithmetic
 // Own: r and d as stored; X: the solution's increment (float-float, FP32) or the
 // solution (FP64); Sum: a thread's or warp's part of a dot product.
-__device__ __forceinline__ FFAcc warp_sum(FFAcc s) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        FFAcc x;
-        x.s = __shfl_xor_sync(0xffffffffu, s.s, o);
-        x.e = __shfl_xor_sync(0xffffffffu, s.e, o);
-        ff_merge(s, x);
-    }
-    return s;
-}
+__device__ __forceinline__ FFAcc warp_sum(FFAcc s) { return ff_warp_sum(s); }
 __device__ __forceinline__ double warp_sum(double s) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -100,19 +91,6 @@ struct CgOps {  // FP32 arithmetic, vectors stored as A::T
         return A::store_val(a, 0);
     }
     static __device__ __forceinline__ float2 up(T v) { return ld_vec(&v); }
-    // ad = m2 d - acc; part of d^dag ad
-    static __device__ __forceinline__ void apply(typename A::Acc& acc, const T (&d)[3], double, float2 m2, T (&ad)[3],
-                                                 Sum& s) {
-        double dot = 0.0;
-#pragma unroll
-        for (int c = 0; c < 2; ++c) ad[c] = A::epilogue(acc, c, up(d[c]), 0.0, m2, dot);
-        // the third row by hand: its epilogue would convert the sum to FP64
-        const float2 sv = up(d[2]), o = make_float2(fmaf(m2.x, sv.x, -acc.c[2].x), fmaf(m2.x, sv.y, -acc.c[2].y));
-        acc.dot = fmaf(sv.x, o.x, acc.dot);
-        acc.dot = fmaf(sv.y, o.y, acc.dot);
-        ad[2] = round(o);
-        s = FFAcc{acc.dot, 0.f};
-    }
     static __device__ __forceinline__ void update_xr(const StepScalars& k, const T (&d)[3], const T (&ad)[3], X (&x)[3],
                                                      T (&r)[3], Sum& s) {
         const float alpha = k.alpha_ff.x;
@@ -144,17 +122,6 @@ struct CgOps<ArithFF> {
     using Sum = FFAcc;
     static constexpr bool kLow = false;
     static __device__ __forceinline__ Sum zero() { return ff_zero(); }
-    static __device__ __forceinline__ void apply(ArithFF::Acc& acc, const T (&d)[3], double, float2 m2, T (&ad)[3],
-                                                 Sum& s) {
-        s = ff_zero();
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float2 re = ff_fma(m2, ff_re(d[c]), ff_neg(ff_result(acc.re[c])));
-            const float2 im = ff_fma(m2, ff_im(d[c]), ff_neg(ff_result(acc.im[c])));
-            ad[c] = ff_cplx(re, im);
-            ff_redot_acc(s, d[c], ad[c]);
-        }
-    }
     static __device__ __forceinline__ void update_xr(const StepScalars& k, const T (&d)[3], const T (&ad)[3], X (&x)[3],
                                                      T (&r)[3], Sum& s) {
         s = ff_zero();
@@ -174,12 +141,6 @@ struct CgOps<ArithF64> {
     using Sum = double;
     static constexpr bool kLow = false;
     static __device__ __forceinline__ Sum zero() { return 0.0; }
-    static __device__ __forceinline__ void apply(ArithF64::Acc& acc, const T (&d)[3], double m2, float2, T (&ad)[3],
-                                                 Sum& s) {
-        s = 0.0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) ad[c] = ArithF64::epilogue(acc, c, d[c], m2, make_float2(0.f, 0.f), s);
-    }
     static __device__ __forceinline__ void update_xr(const StepScalars& k, const T (&d)[3], const T (&ad)[3], X (&x)[3],
                                                      T (&r)[3], Sum& s) {
         s = 0.0;
@@ -211,14 +172,15 @@ struct ResidentParams {
     int fold;   // float-float: iterations between additions of the increment to x
 };
 
-// Threads of a block at most: 64 registers a thread for FP32 arithmetic, 128 else.
+// Threads of a block at most.  FP32 arithmetic takes 1024 (64 registers a thread) where
+// 512 (128 registers) do not reach, the others 512.
 template <class A>
 constexpr int resident_threads() {
     return std::is_same<typename A::C, float2>::value ? 1024 : 512;
 }
 
-template <class A, int NAIK, int S>
-__global__ void __launch_bounds__(resident_threads<A>(), 1) resident_kernel(const ResidentParams<A> p) {
+template <class A, int NAIK, int S, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentParams<A> p) {
     using Ops = CgOps<A>;
     using T = typename A::T;
     using X = typename Ops::X;
@@ -341,7 +303,11 @@ __global__ void __launch_bounds__(resident_threads<A>(), 1) resident_kernel(cons
         {
             typename A::Acc acc;
             lane_site<A, NAIK, S>(p.f, 0, p.t, i, xe, y, z, t, part, active, acc);
-            if (own) Ops::apply(acc, d, m2, m2_ff, ad, s);
+            if (own) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) ad[c] = A::epilogue(acc, c, ld_vec(&d[c]), m2, m2_ff);
+                s = A::dot(acc);
+            }
         }
         s = warp_sum(s);
         exchange(true, lane == 0 ? sum_value(s) : 0.0, [&](double total) {
@@ -473,8 +439,11 @@ cudaError_t launch_lanes(ResidentParams<A> p, int sms, cudaStream_t s) {
     const int per = resident_warps(p.f.g.vh, S, sms);
     const int blocks = (warps + per - 1) / per;
     void* args[] = {&p};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(resident_kernel<A, NAIK, S>), dim3(blocks),
-                                       dim3(32 * per), args, 0, s);
+    const void* kernel = reinterpret_cast<const void*>(resident_kernel<A, NAIK, S, 512>);
+    if constexpr (resident_threads<A>() > 512 && S < 8) {  // eight lanes are taken up to 8 warps only
+        if (32 * per > 512) kernel = reinterpret_cast<const void*>(resident_kernel<A, NAIK, S, 1024>);
+    }
+    return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(32 * per), args, 0, s);
 }
 
 template <class A, int NAIK>

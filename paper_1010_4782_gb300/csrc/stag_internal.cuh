@@ -137,16 +137,16 @@ __device__ __forceinline__ double block_sum(double v, double* smem) {
     return v;
 }
 
-// Each block writes its partial; the last block to finish sums all partials
-// in block order and returns true in every one of its threads, with the total
-// in *total (valid in all threads of that block).  Other blocks return false.
+// v: the block's sum in thread 0.  Each block writes it to partials; the last block to
+// finish sums all of them in block order and returns true in every one of its
+// threads, with the total in *total (valid in all threads of that block).
+// Other blocks return false.
 template <int BS>
-__device__ __forceinline__ bool grid_sum_last_block(double v, double* partials, unsigned int* counter,
-                                                    double* total) {
+__device__ __forceinline__ bool grid_total_last_block(double v, double* partials, unsigned int* counter,
+                                                      double* total) {
     __shared__ double smem[BS / 32];
     __shared__ bool is_last;
     __shared__ double result;
-    v = block_sum<BS>(v, smem);
     if (threadIdx.x == 0) {
         partials[blockIdx.x] = v;
         __threadfence();
@@ -158,7 +158,6 @@ __device__ __forceinline__ bool grid_sum_last_block(double v, double* partials, 
     __threadfence();
     double s = 0.0;
     for (int b = threadIdx.x; b < (int)gridDim.x; b += BS) s += __ldcg(partials + b);
-    __syncthreads();  // smem reuse
     s = block_sum<BS>(s, smem);
     if (threadIdx.x == 0) {
         result = s;
@@ -167,6 +166,14 @@ __device__ __forceinline__ bool grid_sum_last_block(double v, double* partials, 
     __syncthreads();
     *total = result;
     return true;
+}
+
+// The same from a value per thread.
+template <int BS>
+__device__ __forceinline__ bool grid_sum_last_block(double v, double* partials, unsigned int* counter,
+                                                    double* total) {
+    __shared__ double smem[BS / 32];
+    return grid_total_last_block<BS>(block_sum<BS>(v, smem), partials, counter, total);
 }
 
 // ------------------------------------------------------ launch helpers

@@ -26,7 +26,8 @@ struct LinkSet {
 
 // ---- packing (pack.cu)
 // AoS links [Lt][Lz][Ly][Lx][4][3][3] complex128 (device) -> SoA with eta folded,
-// in FP64 and, where the pointer is not null, float-float, FP32, FP16 and BF16.
+// in FP64 and, where the pointer is not null, float-float ([2][4][9][vs]), FP32, FP16 and
+// BF16 (the words of links.cuh).
 void launch_pack_links(const Geom& g, const double* aos, double2* soa64, float4* soaff,
                        float2* soa32, __half2* soa16, __nv_bfloat162* soab16, cudaStream_t s);
 // AoS links -> float-float [2][4][6][vs]: the first two rows, eta folded
@@ -34,7 +35,7 @@ void launch_pack_links_ff_rows2(const Geom& g, const double* aos, float4* soaff_
 // max over the AoS links L of |L^dag L / c^2 - 1| and |det L / c^3 - 1| into *maxdev
 // (a float's bits in an unsigned int, zeroed by the caller)
 void launch_check_scaled_su3(const Geom& g, const double* aos, double c, unsigned int* maxdev, cudaStream_t s);
-// AoS links -> FP32 [2][4][6][vs]: the first two rows, eta folded (12-parameter form)
+// AoS links -> FP32, the first two rows in the words of links.cuh, eta folded (12-parameter form)
 void launch_pack_links_rows2(const Geom& g, const double* aos, float2* soa32r, cudaStream_t s);
 // ABI vector [vh][3] complex128 (device) <-> F64 SoA [3][vs]
 void launch_pack_vec(const Geom& g, const double* aos, double2* soa, cudaStream_t s);
@@ -71,7 +72,7 @@ void launch_dslash_list(bool ff, Epilogue epi, const SysDirac* sys, const int* l
                         const int* count, int grid, cudaStream_t s);
 
 // low-precision Dirac kernels of the mixed-precision solver (same epilogues);
-// lng_inv_scale != 0: the FP32 Naik links are two rows per link ([2][4][6][vs],
+// lng_inv_scale != 0: the FP32 Naik links are two rows per link (links.cuh,
 // eta folded) of scale x SU(3), lng_inv_scale = 1 / scale, the third row rebuilt
 void launch_dslash_f32(const Geom& g, int out_parity, const float2* fat, const float2* lng,
                        const float2* in, float2* out, Epilogue epi, const float2* src, double m2,
@@ -79,7 +80,7 @@ void launch_dslash_f32(const Geom& g, int out_parity, const float2* fat, const f
 void launch_dslash_h16(const Geom& g, int out_parity, const __half2* fat, const __half2* lng,
                        const __half2* in, __half2* out, Epilogue epi, const __half2* src, double m2,
                        CgScalars* scal, double* partials, cudaStream_t s);
-// FP32 with 12-parameter links ([2][4][6][vs], one-hop only): row 2 rebuilt in the kernel
+// FP32 with 12-parameter links (two rows in words, one-hop only): row 2 rebuilt in the kernel
 void launch_dslash_f32r12(const Geom& g, int out_parity, const float2* fat_rows2, const float2* in, float2* out,
                           Epilogue epi, const float2* src, double m2, CgScalars* scal, double* partials,
                           cudaStream_t s);
