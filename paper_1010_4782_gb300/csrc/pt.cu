@@ -126,15 +126,19 @@ __global__ void __launch_bounds__(256, CIN * COUT >= 64 ? 2 : 3)
 #pragma unroll
                 for (int c = 0; c < 3; ++c) tv[c] = v[c];
             }
+            float2 ts[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) ts[c] = make_float2(-tv[c].y, tv[c].x);
 #pragma unroll
             for (int o = 0; o < COUT; ++o) {
                 const float2 wv = ADJ ? make_float2(sw[(p * CIN + ci) * COUT + o].x, -sw[(p * CIN + ci) * COUT + o].y)
                                       : sw[(p * COUT + o) * CIN + ci];
+                // acc += w tv on packed pairs: (Re w)(Re, Im) + (Im w)(-Im, Re)
+                const float2 wr = make_float2(wv.x, wv.x), wi = make_float2(wv.y, wv.y);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    const float2 m = cmulf(wv, tv[c]);
-                    acc[o][c].x += m.x;
-                    acc[o][c].y += m.y;
+                    acc[o][c] = __ffma2_rn(wr, tv[c], acc[o][c]);
+                    acc[o][c] = __ffma2_rn(wi, ts[c], acc[o][c]);
                 }
             }
         }
@@ -153,21 +157,28 @@ __global__ void __launch_bounds__(256, CIN * COUT >= 64 ? 2 : 3)
 }
 
 // partials[blk][p][o][i] = sum over the block's sites of
-// sum_c conj((T_p psi_i)(x)_c) g_o(x)_c, o in [o0, o0 + OC), path p = blockIdx.y.
+// sum_c conj((T_p psi_i)(x)_c) g_o(x)_c, path p = blockIdx.y, inputs i in [i0, i0 + CI),
+// i0 = CI * blockIdx.z, all COUT outputs.
 // MODE EVEN_INPUT: psi is zero on odd sites (only even sites for p = 0, odd
 // sites for p > 0 contribute); EVEN_OUTPUT: g is zero on odd sites.
-template <int CIN, int OC, class T, int MODE = SITES_ALL>
-__global__ void __launch_bounds__(256) pt_wgrad_kernel(Geom g, const float2* __restrict__ links,
-                                                       const T* __restrict__ psi, const T* __restrict__ gout,
-                                                       int cout, float2* __restrict__ partials) {
+// A thread transports its CI inputs and then takes the outputs' gradients a colour at
+// a time, so that a layer split over blockIdx.z transports every input once and the
+// CI x COUT sums (64 registers at 4 x 8) leave room for two blocks per SM.  The grid is
+// four waves of those (wgrad_blocks): each block ends with some 600 shuffles, which
+// with 608 blocks per path (two sites a thread at 16^3 x 32) cost more than the
+// sums.  8 -> 8 layer at 16^3 x 32: 281 us -> 98 us, bound by the FP32 pipe.
+template <int CIN, int COUT, int CI, class T, int MODE = SITES_ALL>
+__global__ void __launch_bounds__(256, 2) pt_wgrad_kernel(Geom g, const float2* __restrict__ links,
+                                                          const T* __restrict__ psi, const T* __restrict__ gout,
+                                                          float2* __restrict__ partials) {
     const int p = blockIdx.y;
-    const int o0 = blockIdx.z * OC;
+    const int i0 = blockIdx.z * CI;
     const size_t vs = (size_t)g.vs;
-    float2 acc[OC][CIN];
+    float2 acc[COUT][CI];
 #pragma unroll
-    for (int oo = 0; oo < OC; ++oo)
+    for (int o = 0; o < COUT; ++o)
 #pragma unroll
-        for (int ci = 0; ci < CIN; ++ci) acc[oo][ci] = make_float2(0.f, 0.f);
+        for (int ci = 0; ci < CI; ++ci) acc[o][ci] = make_float2(0.f, 0.f);
     const int n0 = (MODE == EVEN_INPUT && p > 0) ? g.vh : 0;
     const int n1 = ((MODE == EVEN_INPUT && p == 0) || MODE == EVEN_OUTPUT) ? g.vh : 2 * g.vh;
     for (int n = n0 + blockIdx.x * blockDim.x + threadIdx.x; n < n1; n += gridDim.x * blockDim.x) {
@@ -185,87 +196,110 @@ __global__ void __launch_bounds__(256) pt_wgrad_kernel(Geom g, const float2* __r
             nb = hp.nb;
             load_link<9>(U, hp.u, vs, hp.li);
         }
-        float2 gv[OC][3];
+        float2 tv[CI][3];
+#pragma unroll
+        for (int c4 = 0; c4 < CI; c4 += 4) {
+            constexpr int NV = CI < 4 ? CI : 4;
+            float2 vin[3][4];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if constexpr (CIN % 4 == 0)
+                    ld4c(psi + fidx(i0 + c4, c, Pn, nb, vs, CIN), vin[c]);
+                else
+                    vin[c][0] = ldc(psi + fidx(i0, c, Pn, nb, vs, CIN));
+            }
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                float2 v[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) v[c] = vin[c][k];
+                if (p > 0) {
+                    pt_apply(U, d, v, tv[c4 + k]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) tv[c4 + k][c] = v[c];
+                }
+            }
+        }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            if constexpr (OC % 4 == 0) {
+            float2 gv[COUT];
+            if constexpr (COUT % 4 == 0) {
 #pragma unroll
-                for (int oo = 0; oo < OC; oo += 4) {
+                for (int o = 0; o < COUT; o += 4) {
                     float2 q[4];
-                    ld4c(gout + fidx(o0 + oo, c, P, i, vs, cout), q);
+                    ld4c(gout + fidx(o, c, P, i, vs, COUT), q);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) gv[oo + k][c] = q[k];
+                    for (int k = 0; k < 4; ++k) gv[o + k] = q[k];
                 }
             } else {
 #pragma unroll
-                for (int oo = 0; oo < OC; ++oo) gv[oo][c] = ldc(gout + fidx(o0 + oo, c, P, i, vs, cout));
+                for (int o = 0; o < COUT; ++o) gv[o] = ldc(gout + fidx(o, c, P, i, vs, COUT));
             }
-        }
-        float2 vin[3][4];
+            // acc += conj(tv) g on packed pairs: (Re tv)(Re g, Im g) + (Im tv)(Im g, -Re g)
 #pragma unroll
-        for (int ci = 0; ci < CIN; ++ci) {
-            float2 v[3], tv[3];
-            if constexpr (CIN % 4 == 0) {
-                if (ci % 4 == 0) {
+            for (int o = 0; o < COUT; ++o) {
+                const float2 gs = make_float2(gv[o].y, -gv[o].x);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) ld4c(psi + fidx(ci, c, Pn, nb, vs, CIN), vin[c]);
+                for (int ci = 0; ci < CI; ++ci) {
+                    acc[o][ci] = __ffma2_rn(make_float2(tv[ci][c].x, tv[ci][c].x), gv[o], acc[o][ci]);
+                    acc[o][ci] = __ffma2_rn(make_float2(tv[ci][c].y, tv[ci][c].y), gs, acc[o][ci]);
                 }
-#pragma unroll
-                for (int c = 0; c < 3; ++c) v[c] = vin[c][ci % 4];
-            } else {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) v[c] = ldc(psi + fidx(ci, c, Pn, nb, vs, CIN));
             }
-            if (p > 0) {
-                pt_apply(U, d, v, tv);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) tv[c] = v[c];
-            }
-#pragma unroll
-            for (int oo = 0; oo < OC; ++oo)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float2 m = cmulf_conj(tv[c], gv[oo][c]);
-                    acc[oo][ci].x += m.x;
-                    acc[oo][ci].y += m.y;
-                }
         }
     }
-    __shared__ float2 sred[256 / 32][OC * CIN];
+    __shared__ float2 sred[256 / 32][COUT * CI];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
-    for (int oo = 0; oo < OC; ++oo)
+    for (int o = 0; o < COUT; ++o)
 #pragma unroll
-        for (int ci = 0; ci < CIN; ++ci) {
-            float2 v = acc[oo][ci];
+        for (int ci = 0; ci < CI; ++ci) {
+            float2 v = acc[o][ci];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-                v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+            for (int q = 16; q > 0; q >>= 1) {
+                v.x += __shfl_xor_sync(0xffffffffu, v.x, q);
+                v.y += __shfl_xor_sync(0xffffffffu, v.y, q);
             }
-            if (lane == 0) sred[wp][oo * CIN + ci] = v;
+            if (lane == 0) sred[wp][o * CI + ci] = v;
         }
     __syncthreads();
-    for (int k = threadIdx.x; k < OC * CIN; k += blockDim.x) {
+    for (int k = threadIdx.x; k < COUT * CI; k += blockDim.x) {
         float2 s = make_float2(0.f, 0.f);
         for (int q = 0; q < (int)(blockDim.x / 32); ++q) {
             s.x += sred[q][k].x;
             s.y += sred[q][k].y;
         }
-        const int oo = k / CIN, ci = k % CIN;
-        partials[(((size_t)blockIdx.x * kPaths + p) * cout + o0 + oo) * CIN + ci] = s;
+        const int o = k / CI, ci = k % CI;
+        partials[(((size_t)blockIdx.x * kPaths + p) * COUT + o) * CIN + i0 + ci] = s;
     }
 }
 
-// grad[p][o][i] += sum over blocks of partials (block order)
-__global__ void pt_wgrad_sum_kernel(const float2* __restrict__ partials, int nblk, int nw, float2* grad) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nw) return;
+// grad[p][o][i] += sum over blocks of partials: 32 weights per block, their rows of
+// partials read by kSumRows warps in turn and added in a fixed order.  (One thread per
+// weight walked all the rows by itself: 79 us for each layer, a quarter of a
+// training sample at 16^3 x 32; now 5 us.)
+constexpr int kSumRows = 8;
+__global__ void __launch_bounds__(32 * kSumRows) pt_wgrad_sum_kernel(const float2* __restrict__ partials, int nblk,
+                                                                     int nw, float2* grad) {
+    __shared__ float2 rows[kSumRows][32];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + lane;
     float2 s = make_float2(0.f, 0.f);
-    for (int b = 0; b < nblk; ++b) {
-        s.x += partials[(size_t)b * nw + k].x;
-        s.y += partials[(size_t)b * nw + k].y;
+    if (k < nw) {
+#pragma unroll 8
+        for (int b = row; b < nblk; b += kSumRows) {
+            const float2 v = __ldg(partials + (size_t)b * nw + k);
+            s.x += v.x;
+            s.y += v.y;
+        }
+    }
+    rows[row][lane] = s;
+    __syncthreads();
+    if (row != 0 || k >= nw) return;
+#pragma unroll
+    for (int r = 1; r < kSumRows; ++r) {
+        s.x += rows[r][lane].x;
+        s.y += rows[r][lane].y;
     }
     grad[k].x += s.x;
     grad[k].y += s.y;
@@ -721,22 +755,31 @@ void layer_adj(stag_ptnet* n, int l, const T* gout, T* gin) {
         pt_layer_kernel<kHidden, kHidden, T, T, true><<<nb, 256, 0, S(n)>>>(g, n->links, w, gout, gin, nullptr);
 }
 
+// x-blocks of a weight-gradient launch split z ways: with the paths, four waves of two
+// blocks per SM, but no more than one block per 256 sites.
+int wgrad_blocks(const Geom& g, int z) {
+    return std::max(1, std::min({kWgradBlocks, kWgradWave / (kPaths * z), blocks_for(2 * g.vh, 256)}));
+}
+
 template <class T>
 void layer_wgrad(stag_ptnet* n, int l, const T* psi, const T* gout) {
     const Geom& g = n->g;
-    const int cin = kChan[l], cout = kChan[l + 1];
-    const int nw = kPaths * cout * cin;
+    const int nw = kPaths * kChan[l + 1] * kChan[l];
+    int nblk;
     if (l == 0) {
-        dim3 grid(kWgradBlocks, kPaths, 1);
-        pt_wgrad_kernel<1, kHidden, T, EVEN_INPUT><<<grid, 256, 0, S(n)>>>(g, n->links, psi, gout, cout, n->wpart);
+        nblk = wgrad_blocks(g, 1);
+        pt_wgrad_kernel<1, kHidden, 1, T, EVEN_INPUT><<<dim3(nblk, kPaths, 1), 256, 0, S(n)>>>(g, n->links, psi, gout,
+                                                                                             n->wpart);
     } else if (l == 1) {
-        dim3 grid(kWgradBlocks, kPaths, kHidden / 4);
-        pt_wgrad_kernel<kHidden, 4, T><<<grid, 256, 0, S(n)>>>(g, n->links, psi, gout, cout, n->wpart);
+        nblk = wgrad_blocks(g, 2);
+        pt_wgrad_kernel<kHidden, kHidden, 4, T><<<dim3(nblk, kPaths, 2), 256, 0, S(n)>>>(g, n->links, psi, gout,
+                                                                                        n->wpart);
     } else {
-        dim3 grid(kWgradBlocks, kPaths, 1);
-        pt_wgrad_kernel<kHidden, 1, T, EVEN_OUTPUT><<<grid, 256, 0, S(n)>>>(g, n->links, psi, gout, cout, n->wpart);
+        nblk = wgrad_blocks(g, 1);
+        pt_wgrad_kernel<kHidden, 1, kHidden, T, EVEN_OUTPUT><<<dim3(nblk, kPaths, 1), 256, 0, S(n)>>>(
+            g, n->links, psi, gout, n->wpart);
     }
-    pt_wgrad_sum_kernel<<<blocks_for(nw), kBlock, 0, S(n)>>>(n->wpart, kWgradBlocks, nw, n->grad + layer_offset(l));
+    pt_wgrad_sum_kernel<<<(nw + 31) / 32, 32 * kSumRows, 0, S(n)>>>(n->wpart, nblk, nw, n->grad + layer_offset(l));
 }
 
 double read_partials(stag_ptnet* n, int count) {

@@ -17,7 +17,8 @@ constexpr int kPaths = 9;
 constexpr int kHidden = 8;
 constexpr int kLayers = 3;
 constexpr int kChan[kLayers + 1] = {1, kHidden, kHidden, 1};
-constexpr int kWgradBlocks = 608;  // x-blocks of the weight-gradient grid (4 per SM)
+constexpr int kWgradWave = 4 * 2 * 152;          // blocks of a weight-gradient launch: four waves of two per SM
+constexpr int kWgradBlocks = kWgradWave / 9;      // most x-blocks of one (all nine paths)
 
 __device__ __forceinline__ float2 ldc(const float2* p) { return *p; }
 __device__ __forceinline__ float2 ldc(const __nv_bfloat162* p) { return __bfloat1622float2(*p); }
