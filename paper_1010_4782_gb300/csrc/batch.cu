@@ -94,7 +94,9 @@ struct stag_batch {
     double* io_b = nullptr;
     MultiGroup* d_groups = nullptr;
     int4* d_items = nullptr;
-    std::vector<std::pair<Tune, std::pair<int, int>>> classes;  // (tuning, [first item, count))
+    using LaunchClass = std::pair<Tune, std::pair<int, int>>;  // (shape, [first item, count))
+    std::vector<LaunchClass> classes;      // of the Dirac kernels
+    std::vector<LaunchClass> vec_classes;  // of the vector steps
     CgScalars* scal = nullptr;       // one per system
     CgScalars* aux = nullptr;        // scratch reductions
     CgScalars* scal_host = nullptr;  // pinned, n_sys + 1
@@ -199,43 +201,91 @@ MultiLaunch make_launch(stag_batch* b, int parity, int phase, int first_item) {
 // block (16384 blocks), 3.48 s with 4096 blocks and 3.60 s with 2048.
 constexpr int kMaxGroupBlocks = 4096;
 
-// Blocks of a group for a shape: one per tile of sites, at most kMaxGroupBlocks
-// (blocks then take contiguous runs of tiles); for the resident sweep, at most
-// the number of blocks of that shape the GPU holds at once.
-int group_blocks(const Group& G, int rb, int bs, int mode) {
-    const int spb = bs / (G.rpad / rb);
-    const int ntiles = (G.g.vh + spb - 1) / spb;
-    int cap = kMaxGroupBlocks;
-    if (mode) {
-        int dev = 0, sms = 1;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cap = std::min(cap, multi_resident_blocks_per_sm(rb, bs) * sms);
+int sm_count() {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// Blocks of each of the groups gis in one launch of a shape.  Contiguous runs: one per
+// tile of sites, at most kMaxGroupBlocks.  Resident sweep: `resident` blocks (those the GPU
+// holds at once) for every group, or (shared) divided among the groups in proportion to
+// their tiles.  The Dirac kernels take the former: with ten lattices of three sizes in a
+// launch the many short blocks balance better (D_oe 79 us against 106 shared).  The
+// vector steps, whose blocks are dominated by their reduction, fence and ticket, the latter.
+std::vector<int> launch_blocks(stag_batch* b, const std::vector<int>& gis, int rb, int bs, int mode, int resident,
+                               bool shared) {
+    std::vector<int> n;
+    long long total = 0;
+    for (int gi : gis) {
+        const Group& G = b->groups[gi];
+        const int spb = bs / (G.rpad / rb);
+        n.push_back((G.g.vh + spb - 1) / spb);
+        total += n.back();
     }
-    return std::min(ntiles, cap);
+    for (int& t : n) {
+        long long cap = mode ? resident : kMaxGroupBlocks;
+        if (mode && shared) cap = std::max<long long>(1, (cap * t + total - 1) / total);
+        t = (int)std::min<long long>(t, std::min<long long>(cap, kMaxGroupBlocks));
+    }
+    return n;
 }
 
 void add_items(std::vector<int4>& v, int gi, int nblk, int mode) {
     for (int k = 0; k < nblk; ++k) v.push_back(make_int4(gi, k, nblk, mode));
 }
 
-// Work items of every group with its tuned shape, grouped into launch classes.
+void add_launch(stag_batch* b, std::vector<int4>& v, const std::vector<int>& gis, int rb, int bs, int mode,
+                int resident, bool shared) {
+    const std::vector<int> n = launch_blocks(b, gis, rb, bs, mode, resident, shared);
+    for (size_t q = 0; q < gis.size(); ++q) add_items(v, gis[q], n[q], mode);
+}
+
+// Shape of the vector steps of single-right-hand-side groups: whole blocks of 256 threads, as
+// many as the GPU holds at once.  (In the Dirac kernel's shape, e.g. 64 threads and a
+// reduction for every two tiles, the x/r update of a ten-system batch took 43 us and the
+// d update 20 us; now 29 and 14 us.)
+constexpr int kVecBlock = 256;
+constexpr int kVecBlocksPerSm = 8;
+
+// Work items of every group with its tuned shape, grouped into launch classes, for the
+// Dirac kernels and (classes marked vec) for the vector steps.
 void build_items(stag_batch* b) {
-    std::map<std::tuple<int, int, int>, std::vector<int4>> by_class;
+    std::map<std::tuple<int, int, int>, std::vector<int>> by_class;
+    std::vector<int> singles;
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
         const Group& G = b->groups[gi];
-        add_items(by_class[{G.tune.rb, G.tune.bs, G.tune.mode}], (int)gi,
-                  group_blocks(G, G.tune.rb, G.tune.bs, G.tune.mode), G.tune.mode);
+        by_class[{G.tune.rb, G.tune.bs, G.tune.mode}].push_back((int)gi);
+        if (G.nrhs == 1) singles.push_back((int)gi);
     }
     std::vector<int4> all;
     b->classes.clear();
+    b->vec_classes.clear();
+    auto add_class = [&](std::vector<stag_batch::LaunchClass>& to, const Tune& t, const std::vector<int>& gis,
+                         int resident, bool shared) {
+        const int first = (int)all.size();
+        add_launch(b, all, gis, t.rb, t.bs, t.mode, resident, shared);
+        to.push_back({t, {first, (int)all.size() - first}});
+    };
     for (auto& kv : by_class) {
         Tune t;
         t.rb = std::get<0>(kv.first);
         t.bs = std::get<1>(kv.first);
         t.mode = std::get<2>(kv.first);
-        b->classes.push_back({t, {(int)all.size(), (int)kv.second.size()}});
-        all.insert(all.end(), kv.second.begin(), kv.second.end());
+        const int resident = t.mode ? multi_resident_blocks_per_sm(t.rb, t.bs) * sm_count() : 0;
+        add_class(b->classes, t, kv.second, resident, false);
+        std::vector<int> multi;
+        for (int gi : kv.second)
+            if (b->groups[gi].nrhs > 1) multi.push_back(gi);
+        if (!multi.empty()) add_class(b->vec_classes, t, multi, resident, false);
+    }
+    if (!singles.empty()) {
+        Tune t;
+        t.rb = 1;
+        t.bs = kVecBlock;
+        t.mode = 1;
+        add_class(b->vec_classes, t, singles, kVecBlocksPerSm * sm_count(), true);
     }
     if (b->d_items) cudaFree(b->d_items);
     b->d_items = nullptr;
@@ -250,7 +300,8 @@ void build_items(stag_batch* b) {
 }
 
 void enqueue_all(stag_batch* b, MultiKernel k, int parity, int phase) {
-    for (auto& c : b->classes)
+    const bool vec = k == MK_UPDATE_XR || k == MK_UPDATE_D;
+    for (auto& c : vec ? b->vec_classes : b->classes)
         launch_multi(k, make_launch(b, parity, phase, c.second.first), c.second.second, c.first.rb, c.first.bs,
                      c.first.mode, b->s);
 }
@@ -313,7 +364,7 @@ void store_tune(const std::string& key, const Tune& t) {
 // group whose systems are all done returns at once).
 std::pair<double, double> time_group_launch(stag_batch* b, const std::vector<int>& gis, int rb, int bs, int mode) {
     std::vector<int4> items;
-    for (int gi : gis) add_items(items, gi, group_blocks(b->groups[gi], rb, bs, mode), mode);
+    add_launch(b, items, gis, rb, bs, mode, mode ? multi_resident_blocks_per_sm(rb, bs) * sm_count() : 0, false);
     int4* d_items = nullptr;
     bcheck(b, cudaMalloc(&d_items, items.size() * sizeof(int4)), "allocate tuning items");
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // D_oe start, end; D_eo start, end
