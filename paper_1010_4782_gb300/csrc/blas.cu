@@ -269,15 +269,6 @@ __global__ void __launch_bounds__(kBlock) to_ff_kernel(Geom g, const double2* __
     for (int c = 0; c < 3; ++c) out[c * vs + i] = ff_from_complex(in[c * vs + i]);
 }
 
-__global__ void __launch_bounds__(kBlock) from_ff_kernel(Geom g, const float4* __restrict__ in,
-                                                         double2* __restrict__ out) {
-    const int i = blockIdx.x * kBlock + threadIdx.x;
-    if (i >= g.vs) return;
-    const size_t vs = (size_t)g.vs;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) out[c * vs + i] = ff_to_complex(in[c * vs + i]);
-}
-
 // ------------------------------------------------------------ launchers
 int resident_wave_blocks() {
     static std::atomic<int> cached[64];  // per device ordinal; 0 = not yet queried
@@ -339,10 +330,6 @@ void launch_norm2_diff(const Geom& g, const double2* a, const double2* b, CgScal
 
 void launch_to_ff(const Geom& g, const double2* in, float4* out, cudaStream_t s) {
     to_ff_kernel<<<blocks_for(g.vs), kBlock, 0, s>>>(g, in, out);
-}
-
-void launch_from_ff(const Geom& g, const float4* in, double2* out, cudaStream_t s) {
-    from_ff_kernel<<<blocks_for(g.vs), kBlock, 0, s>>>(g, in, out);
 }
 
 }  // namespace stag

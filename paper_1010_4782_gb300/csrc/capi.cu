@@ -970,22 +970,20 @@ int stag_dslash(stag_handle* h, int32_t out_parity, const double* in, double* ou
         const Geom& g = h->g;
         const bool out_dev = is_device_ptr(h, out);
         const double* src = input_vec(h, in, h->io_a);
-        launch_pack_vec(g, src, h->x, h->s);
+        double* dst = out_dev ? out : h->io_b;
         if (use_ff(h)) {
             float4* in_ff = reinterpret_cast<float4*>(h->u);
-            launch_to_ff(g, h->x, in_ff, h->s);
+            launch_pack_vec_ff(g, src, in_ff, h->s);
             launch_dslash_ff(g, out_parity, links(h), in_ff, static_cast<float4*>(h->t), EPI_PLAIN,
                              nullptr, 0.0, nullptr, nullptr, h->s);
-            launch_from_ff(g, static_cast<const float4*>(h->t), h->ad, h->s);
-            h->launches += 3;
+            launch_unpack_vec_ff(g, static_cast<const float4*>(h->t), dst, h->s);
         } else {
+            launch_pack_vec(g, src, h->x, h->s);
             launch_dslash_f64(g, out_parity, links(h), h->x, h->ad, EPI_PLAIN, nullptr, 0.0, nullptr,
                               nullptr, h->s);
-            h->launches += 1;
+            launch_unpack_vec(g, h->ad, dst, h->s);
         }
-        double* dst = out_dev ? out : h->io_b;
-        launch_unpack_vec(g, h->ad, dst, h->s);
-        h->launches += 2;
+        h->launches += 3;
         launch_check(h, "dslash");
         if (!out_dev)
             cuda_check(h, cudaMemcpyAsync(out, h->io_b, abi_vec_bytes(g), cudaMemcpyDeviceToHost, h->s),
@@ -1010,23 +1008,22 @@ int stag_apply_A(stag_handle* h, const double* in_even, double* out_even) {
         const Geom& g = h->g;
         const bool out_dev = is_device_ptr(h, out_even);
         const double* src = input_vec(h, in_even, h->io_a);
-        launch_pack_vec(g, src, h->x, h->s);
-        const double m2 = h->mass * h->mass;
+        double* dst = out_dev ? out_even : h->io_b;
         if (use_ff(h)) {
             float4* in_ff = reinterpret_cast<float4*>(h->u);
-            launch_to_ff(g, h->x, in_ff, h->s);
             float4* t = static_cast<float4*>(h->t);
             float4* out_ff = reinterpret_cast<float4*>(h->r);
+            launch_pack_vec_ff(g, src, in_ff, h->s);
             launch_dslash_ff(g, 1, links(h), in_ff, t, EPI_PLAIN, nullptr, 0.0, nullptr, nullptr, h->s);
-            launch_dslash_ff(g, 0, links(h), t, out_ff, EPI_AXPY, in_ff, m2, nullptr, nullptr, h->s);
-            launch_from_ff(g, out_ff, h->ad, h->s);
+            launch_dslash_ff(g, 0, links(h), t, out_ff, EPI_AXPY, in_ff, h->mass * h->mass, nullptr, nullptr, h->s);
+            launch_unpack_vec_ff(g, out_ff, dst, h->s);
             h->launches += 4;
         } else {
+            launch_pack_vec(g, src, h->x, h->s);
             apply_A_f64(h, h->x, h->ad);
+            launch_unpack_vec(g, h->ad, dst, h->s);
+            h->launches += 2;
         }
-        double* dst = out_dev ? out_even : h->io_b;
-        launch_unpack_vec(g, h->ad, dst, h->s);
-        h->launches += 2;
         launch_check(h, "apply_A");
         if (!out_dev)
             cuda_check(h, cudaMemcpyAsync(out_even, h->io_b, abi_vec_bytes(g), cudaMemcpyDeviceToHost, h->s),

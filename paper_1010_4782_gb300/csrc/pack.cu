@@ -182,6 +182,36 @@ __global__ void __launch_bounds__(kBlock) unpack_vec_kernel(Geom g, const double
     for (int c = 0; c < 3; ++c) aos[(size_t)i * 3 + c] = soa[c * vs + i];
 }
 
+// ABI vector <-> float-float SoA in one pass each way.  Through FP64 SoA it was two, and
+// stag_apply_A in float-float at 32^3 x 64 took 941 us; with these two kernels (19 and 20 us,
+// 100 MB each) it takes 858, 818 of them in the two hops.
+__global__ void __launch_bounds__(kBlock) pack_vec_ff_kernel(Geom g, const double2* __restrict__ aos,
+                                                             float4* __restrict__ soa) {
+    const int i = blockIdx.x * kBlock + threadIdx.x;
+    if (i >= g.vs) return;
+    const size_t vs = (size_t)g.vs;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        soa[c * vs + i] = i < g.vh ? ff_from_complex(aos[(size_t)i * 3 + c]) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+__global__ void __launch_bounds__(kBlock) unpack_vec_ff_kernel(Geom g, const float4* __restrict__ soa,
+                                                               double2* __restrict__ aos) {
+    const int i = blockIdx.x * kBlock + threadIdx.x;
+    if (i >= g.vh) return;
+    const size_t vs = (size_t)g.vs;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) aos[(size_t)i * 3 + c] = ff_to_complex(soa[c * vs + i]);
+}
+
+void launch_pack_vec_ff(const Geom& g, const double* aos, float4* soa, cudaStream_t s) {
+    pack_vec_ff_kernel<<<blocks_for(g.vs), kBlock, 0, s>>>(g, reinterpret_cast<const double2*>(aos), soa);
+}
+
+void launch_unpack_vec_ff(const Geom& g, const float4* soa, double* aos, cudaStream_t s) {
+    unpack_vec_ff_kernel<<<blocks_for(g.vh), kBlock, 0, s>>>(g, soa, reinterpret_cast<double2*>(aos));
+}
+
 void launch_pack_vec(const Geom& g, const double* aos, double2* soa, cudaStream_t s) {
     pack_vec_kernel<<<blocks_for(g.vs), kBlock, 0, s>>>(g, reinterpret_cast<const double2*>(aos), soa);
 }

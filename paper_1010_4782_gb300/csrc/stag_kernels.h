@@ -40,6 +40,9 @@ void launch_pack_links_rows2(const Geom& g, const double* aos, float2* soa32r, c
 // ABI vector [vh][3] complex128 (device) <-> F64 SoA [3][vs]
 void launch_pack_vec(const Geom& g, const double* aos, double2* soa, cudaStream_t s);
 void launch_unpack_vec(const Geom& g, const double2* soa, double* aos, cudaStream_t s);
+// ABI vector <-> float-float SoA
+void launch_pack_vec_ff(const Geom& g, const double* aos, float4* soa, cudaStream_t s);
+void launch_unpack_vec_ff(const Geom& g, const float4* soa, double* aos, cudaStream_t s);
 
 // ---- Dirac kernels (dslash.cu)
 void launch_dslash_f64(const Geom& g, int out_parity, const LinkSet& L, const double2* in,
@@ -172,8 +175,7 @@ void launch_from_lo(const Geom& g, const V* in, double2* out, double scale, cuda
 // x += sigma * y (FP64); y = 0
 void launch_lo_fold_y(const Geom& g, double2* x, float2* y, double sigma, cudaStream_t s);
 
-// F64 SoA vector <-> FF SoA vector
+// F64 SoA vector -> FF SoA vector
 void launch_to_ff(const Geom& g, const double2* in, float4* out, cudaStream_t s);
-void launch_from_ff(const Geom& g, const float4* in, double2* out, cudaStream_t s);
 
 }  // namespace stag
