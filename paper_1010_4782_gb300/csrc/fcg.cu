@@ -62,7 +62,6 @@ struct Arith<float4> {
         ff_mac(a, z.x, 0.f, v.x, v.y);
         ff_mac(a, z.y, 0.f, v.z, v.w);
     }
-    static __device__ __forceinline__ double total(const Acc& a) { return ff_acc_to_double(a); }
     // s a + b, the scalar given in FP64 and as a float-float pair
     static __device__ __forceinline__ float4 axpy(double, float2 s, float4 a, float4 b) { return ff_caxpy(s, a, b); }
     static __device__ __forceinline__ float4 from_z(float2 z) { return make_float4(z.x, 0.f, z.y, 0.f); }
@@ -79,7 +78,6 @@ struct Arith<double2> {
     static __device__ __forceinline__ void zdot(Acc& a, float2 z, double2 v) {
         a = fma((double)z.x, v.x, fma((double)z.y, v.y, a));
     }
-    static __device__ __forceinline__ double total(const Acc& a) { return a; }
     static __device__ __forceinline__ double2 axpy(double s, float2, double2 a, double2 b) {
         return make_double2(fma(s, a.x, b.x), fma(s, a.y, b.y));
     }
@@ -89,17 +87,24 @@ struct Arith<double2> {
     static __device__ __forceinline__ float2 f2(double2 v) { return make_float2((float)v.x, (float)v.y); }
 };
 
+// A block's sum (thread 0).  Float-float values stay float-float, as wide as the threads'
+// sums: FP64 adds run at two lanes per cycle and SM, and the shuffles' two FP64 sums took
+// 10 of fcg_out_kernel's 48 us at 24^3 x 48.
+__device__ __forceinline__ double block_total(double v, double* sm) { return block_sum<kBlock>(v, sm); }
+__device__ __forceinline__ double block_total(FFAcc v, double*) { return block_sum<kBlock>(v); }
+
 // Two grid sums at once: per-block partials of a and b, then the last block to
 // finish adds them in block order (deterministic).  True in every thread of
 // that block, with the sums in out[0..1].
-__device__ __forceinline__ bool grid_sum2_last_block(double a, double b, double* partials, unsigned int* counter,
+template <class Acc>
+__device__ __forceinline__ bool grid_sum2_last_block(Acc va, Acc vb, double* partials, unsigned int* counter,
                                                      double* out) {
     __shared__ double sm[kBlock / 32];
     __shared__ bool is_last;
     __shared__ double res[2];
-    a = block_sum<kBlock>(a, sm);
+    const double a = block_total(va, sm);
     __syncthreads();
-    b = block_sum<kBlock>(b, sm);
+    const double b = block_total(vb, sm);
     if (threadIdx.x == 0) {
         partials[2 * blockIdx.x] = a;
         partials[2 * blockIdx.x + 1] = b;
@@ -209,7 +214,7 @@ __global__ void __launch_bounds__(kBlock) fcg_update_kernel(Geom g, V* __restric
         }
     }
     double total;
-    if (grid_sum_last_block<kBlock>(Arith<V>::total(n2), partials, &d->sc.counter, &total)) {
+    if (grid_sum_last_block<kBlock>(n2, partials, &d->sc.counter, &total)) {
         if (threadIdx.x == 0) after_update(d, total);
     }
 }
@@ -249,16 +254,18 @@ __global__ void __launch_bounds__(kBlock) fcg_zdots_kernel(Geom g, const T* __re
         }
     }
     double tot[2];
-    if (grid_sum2_last_block(Arith<V>::total(zr), Arith<V>::total(zq), partials, &d->sc.counter, tot)) {
+    if (grid_sum2_last_block(zr, zq, partials, &d->sc.counter, tot)) {
         if (threadIdx.x == 0) finish_zdots(d, tot, start);
     }
 }
 
 // Collapsed form of the network, fused: z = k0 r + sum_p T_p chi_p on even
 // sites (pt_out_site; chi from pt_chi_kernel), stored in FP32, with (z, r),
-// (z, q) and beta as in fcg_zdots_kernel.
+// (z, q) and beta as in fcg_zdots_kernel.  Latency-bound like pt_chi_kernel: the eight
+// directions unrolled and three blocks an SM (80 registers) 52 -> 46 us at 24^3 x 48, the
+// float-float block sums 38 us (167 MB: 25 us at measured HBM rate); the solve there 129.2 -> 121.4 ms.
 template <class V, class TS, class L>
-__global__ void __launch_bounds__(kBlock) fcg_out_kernel(Geom g, const L* __restrict__ links,
+__global__ void __launch_bounds__(kBlock, 3) fcg_out_kernel(Geom g, const L* __restrict__ links,
                                                          const float2* __restrict__ coef, const TS* __restrict__ chi,
                                                          const V* __restrict__ r, const V* __restrict__ q,
                                                          float2* __restrict__ z, FcgDev* d, double* partials,
@@ -285,7 +292,7 @@ __global__ void __launch_bounds__(kBlock) fcg_out_kernel(Geom g, const L* __rest
         }
     }
     double tot[2];
-    if (grid_sum2_last_block(Arith<V>::total(zr), Arith<V>::total(zq), partials, &d->sc.counter, tot)) {
+    if (grid_sum2_last_block(zr, zq, partials, &d->sc.counter, tot)) {
         if (threadIdx.x == 0) finish_zdots(d, tot, start);
     }
 }

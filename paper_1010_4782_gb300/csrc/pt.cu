@@ -589,16 +589,21 @@ __global__ void pt_collapse_kernel(const float2* __restrict__ w, float2* __restr
     coef[t] = make_float2((float)h.x, (float)h.y);
 }
 
-// chi on odd sites (pt_chi_site), stored as TS; links stored as L
+// chi on odd sites (pt_chi_site), stored as TS; links stored as L.  Bound by the latency of
+// its loads: the 24 sums take 48 registers, so only 16 warps fit an SM.  With the eight
+// directions unrolled the next ones' loads are in flight during a direction's arithmetic:
+// 24^3 x 48, float-float r, 44 -> 34 us (143 MB: 21 us at measured HBM rate).  Blocks of 64
+// threads make the last wave finer than blocks of 256: 32 us.
+constexpr int kChiBlock = 64, kChiBlocksPerSm = 8;
 template <class V, class TS, class L>
-__global__ void __launch_bounds__(256, 2) pt_chi_kernel(Geom g, const L* __restrict__ links,
+__global__ void __launch_bounds__(kChiBlock, kChiBlocksPerSm) pt_chi_kernel(Geom g, const L* __restrict__ links,
                                                         const float2* __restrict__ coef, const V* __restrict__ r,
                                                         TS* __restrict__ chi, const int* __restrict__ skip) {
     if (skip && *skip) return;
     __shared__ float2 sH[64];
     for (int k = threadIdx.x; k < 64; k += blockDim.x) sH[k] = coef[1 + k];
     __syncthreads();
-    const int i = blockIdx.x * 256 + threadIdx.x;
+    const int i = blockIdx.x * kChiBlock + threadIdx.x;
     if (i >= g.vh) return;
     const size_t vs = (size_t)g.vs;
     float2 acc[8][3];
@@ -962,12 +967,12 @@ void pt_collapse(stag_ptnet* n) {
 
 template <class V>
 void launch_pt_chi_any(stag_ptnet* n, const V* r, const int* skip) {
-    const int nb = blocks_for(n->g.vh, 256);
+    const int nb = blocks_for(n->g.vh, kChiBlock);
     if (infer_bf16(n))
-        pt_chi_kernel<V, __nv_bfloat162, __half2><<<nb, 256, 0, S(n)>>>(
+        pt_chi_kernel<V, __nv_bfloat162, __half2><<<nb, kChiBlock, 0, S(n)>>>(
             n->g, n->links16, n->coef, r, static_cast<__nv_bfloat162*>(n->act[2]), skip);
     else
-        pt_chi_kernel<V, float2, float2><<<nb, 256, 0, S(n)>>>(n->g, n->links, n->coef, r,
+        pt_chi_kernel<V, float2, float2><<<nb, kChiBlock, 0, S(n)>>>(n->g, n->links, n->coef, r,
                                                                static_cast<float2*>(n->act[2]), skip);
 }
 void launch_pt_chi(stag_ptnet* n, const float4* r, const int* skip) { launch_pt_chi_any(n, r, skip); }

@@ -153,7 +153,7 @@ __device__ __forceinline__ void pt_chi_site(const Geom& g, const L* __restrict__
     for (int p = 0; p < 8; ++p)
 #pragma unroll
         for (int c = 0; c < 3; ++c) acc[p][c] = make_float2(0.f, 0.f);
-#pragma unroll 1
+#pragma unroll
     for (int q = 1; q < kPaths; ++q) {
         const int mu = (q - 1) >> 1, d = (q - 1) & 1;
         const HopT<L> hp = pt_hop(g, links, 1, i, x, y, z, t, mu, d);
@@ -188,7 +188,7 @@ __device__ __forceinline__ void pt_out_site(const Geom& g, const L* __restrict__
     site_coords(i, 0, g, x, y, z, t);
 #pragma unroll
     for (int c = 0; c < 3; ++c) out[c] = cmulf(k0, r0[c]);
-#pragma unroll 1
+#pragma unroll
     for (int p = 1; p < kPaths; ++p) {
         const int mu = (p - 1) >> 1, d = (p - 1) & 1;
         const HopT<L> hp = pt_hop(g, links, 0, i, x, y, z, t, mu, d);
