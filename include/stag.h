@@ -94,12 +94,17 @@ typedef struct stag_handle stag_handle; /* opaque; owned by the library */
 
 typedef struct {
     int32_t arith;          /* STAG_ARITH_*, Dirac arithmetic of the CG iteration (default F64) */
-    int32_t check_interval; /* CG iterations between host convergence reads (default 32)     */
+    int32_t check_interval; /* CG iterations between host convergence reads (default 32); lattices
+                               small enough for one launch of many iterations (up to about
+                               78,000 sites of a parity in FP64 class, 156,000 in FP32) read
+                               every 512 rounded down to a multiple of it                     */
     int32_t max_restarts;   /* restarts of Fig. 1 from the current x when the true residual
                                exceeds tol (default 5)                                        */
-    int32_t use_graphs;     /* capture check_interval iterations as one CUDA graph (default 1) */
-    int32_t timing;         /* record CUDA events around every CG kernel (default 0);
-                               disables graphs; read with stag_kernel_stats                    */
+    int32_t use_graphs;     /* capture check_interval iterations as one CUDA graph (default 1);
+                               no effect on those small lattices                               */
+    int32_t timing;         /* record CUDA events around every CG kernel (default 0; on those
+                               small lattices the device's clock around every phase of the
+                               launch); disables graphs; read with stag_kernel_stats           */
     int32_t inner;          /* STAG_INNER_*, precision of the CG iteration (default NONE)      */
     int32_t reliable_interval; /* mixed precision: most iterations between residual
                                   replacements (default 100)                                  */
@@ -198,7 +203,8 @@ int stag_apply_A_prec(stag_handle* h, int32_t arith, const double* in_even, doub
  * the true residual is then recomputed with native FP64 arithmetic and Fig. 1
  * restarts from the current x while it exceeds tol (at most max_restarts times).
  * Returns STAG_OK, STAG_ERR_NOT_CONVERGED (x holds the last iterate) or
- * STAG_ERR_BREAKDOWN; info (nullable) is filled in every case. */
+ * STAG_ERR_BREAKDOWN; info (nullable) is filled in every case.  (STAG_ERR_TIMEOUT: a
+ * bounded wait between the blocks of the small lattices' launch ran out.) */
 int stag_cg_solve(stag_handle* h, const double* b_even, double* x_even, double tol,
                   int32_t max_iter, stag_solve_info* info);
 
@@ -209,8 +215,9 @@ int stag_destroy(stag_handle* h);
  * on this thread).  Never NULL; valid until the next call on the handle. */
 const char* stag_last_error(const stag_handle* h);
 
-/* Accumulated CUDA-event time and launch count of one CG kernel (STAG_KERNEL_*),
- * recorded while the handle's timing option is on. */
+/* Accumulated time and launch count of one CG kernel (STAG_KERNEL_*), or of its
+ * phase where the iterations run in one launch, recorded while the handle's timing
+ * option is on. */
 int stag_kernel_stats(const stag_handle* h, int32_t kernel, double* total_ms, int64_t* launches);
 
 /* Zero the kernel statistics. */

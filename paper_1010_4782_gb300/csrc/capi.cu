@@ -3,8 +3,9 @@
 //
 // The driver keeps alpha, beta and delta on the device (the paper's CUBLAS
 // dot returned a scalar to the host every step).  It enqueues blocks of
-// check_interval iterations - captured once as a CUDA graph - and reads the
-// CG state back only between blocks.  After Fig. 1 stops, the true residual
+// check_interval iterations - captured once as a CUDA graph, or for small
+// lattices up to 512 of them in one cooperative launch (resident.cu) - and reads
+// the CG state back only between blocks.  After Fig. 1 stops, the true residual
 // b - A x is recomputed with native FP64 arithmetic and Fig. 1 restarts from
 // the current x while it exceeds tol.
 #include <algorithm>
@@ -321,7 +322,8 @@ constexpr int kResidentIters = 512;
 // Is the iteration's arithmetic FP32 (the mixed-precision inner iteration)?
 bool iterates_in_fp32(const stag_handle* h) { return h->opt.inner != STAG_INNER_NONE; }
 
-void launch_resident(stag_handle* h, int iters) {
+// False if the device cannot hold the grid at once (a context limited to some of the SMs).
+bool launch_resident(stag_handle* h, int iters) {
     const Geom& g = h->g;
     ResidentWork w = h->rwork;
     if (!h->opt.timing) w.ns = nullptr;
@@ -345,18 +347,27 @@ void launch_resident(stag_handle* h, int iters) {
         e = launch_resident_f64(g, links(h), static_cast<double2*>(h->d), static_cast<double2*>(h->t), h->r, h->x,
                                 h->scal, w, iters, h->s);
     }
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return false;
+    }
     cuda_check(h, e, "resident CG launch");
     h->launches += 1;
+    return true;
 }
 
 // Fig. 1 in launches of many iterations each (resident.cu).  A block hook is
-// called every check_interval iterations, as with blocks of launches.
-void run_fig1_resident(stag_handle* h) {
+// called every check_interval iterations, as with blocks of launches.  False, with
+// the state as cg_init left it, if the grid does not fit.
+bool run_fig1_resident(stag_handle* h) {
     const int K = h->opt.check_interval;
     const int iters = h->block_hook ? K : std::max(1, kResidentIters / K) * K;
     long long iter_before = 0;  // a run starts at iteration 0
     do {
-        launch_resident(h, iters);
+        if (!launch_resident(h, iters)) {
+            h->resident = false;
+            return false;
+        }
         read_state(h);
         if (h->block_hook) h->block_hook();
         if (h->opt.timing) {
@@ -372,14 +383,12 @@ void run_fig1_resident(stag_handle* h) {
         }
         iter_before = h->scal_host->iter;
     } while (!h->scal_host->done);
+    return true;
 }
 
 // Runs Fig. 1 from the state prepared by cg_init until scal->done.
 void run_fig1(stag_handle* h) {
-    if (h->resident && resident_fits(h->g, iterates_in_fp32(h))) {
-        run_fig1_resident(h);
-        return;
-    }
+    if (h->resident && resident_fits(h->g, iterates_in_fp32(h)) && run_fig1_resident(h)) return;
     const int K = h->opt.check_interval;
     const bool timing = h->opt.timing != 0;
     const bool graphs = h->opt.use_graphs != 0 && !timing;

@@ -1,6 +1,5 @@
 // dirac.cuh - the arithmetics and single-hop products of the Dirac kernels
-// (dslash.cu: one thread per output site; wave.cu: one thread per output site
-// and direction).
+// (dslash.cu: one thread per output site; dirac_lanes.cuh: one to eight lanes per site).
 #pragma once
 
 #include <cuda_bf16.h>

@@ -14,8 +14,8 @@
 // (8 or 16 reads of each input site) are served by L1/L2: a 28^3 x 96
 // half-lattice FP64 vector is 50.6 MB, well inside the 126 MB L2.
 //
-// Two arithmetics share the kernel body: native FP64 FMA (F64) and
-// float-float on the FP32 pipelines (FF, see ff.cuh).
+// The arithmetics (dirac.cuh: native FP64, float-float on the FP32 pipelines, FP32 on
+// FP32 and 16-bit storage) share the kernel body.
 //
 // Epilogues (used by A = m^2 - D_eo D_oe, Eq. (3)):
 //   EPI_PLAIN  out = D in

@@ -21,8 +21,8 @@
 // alpha, beta and the decision to stop are the same bits in every block.
 //
 // Per iteration, before (four launches in a graph) and now: 4^4 one-hop FP64 38 -> 14.6
-// us, 8^3 x 16 float-float 50 -> 15.2, FP64 91 -> 23.5, 16^4 one-hop FP32 26 -> 19,
-// 20 x 18 x 14 x 30 FP32 43 -> 34 (solve times over iterations, reliable updates
+// us, 8^3 x 16 float-float 50 -> 15.2, FP64 91 -> 23.5, 16^4 one-hop FP32 26 -> 17.6,
+// 20 x 18 x 14 x 30 FP32 43 -> 32.5 (solve times over iterations, reliable updates
 // included), 16^3 x 32 float-float 104 -> 66.  Bound now: the exchanges and the FP64
 // scalars below 10,000 sites (about 9 us of an iteration), L2 and the FP32 or FP64
 // pipes above.
