@@ -436,7 +436,6 @@ void destroy_handle(stag_handle* h) {
     for (const stag_handle::Alloc& a : h->allocs) cudaFree(a.base);
     h->allocs.clear();
     if (h->scal_host) cudaFreeHost(h->scal_host);
-    if (h->timeout_host) cudaFreeHost(h->timeout_host);
     if (h->ev_in) cudaEventDestroy(h->ev_in);
     if (h->s) cudaStreamDestroy(h->s);
     delete h;
@@ -888,19 +887,20 @@ int stag_create_ex(stag_handle** out, const double* fat, const double* naik_long
         // one partial sum per block of any reducing kernel (blocks of 64 threads or more)
         h->partials = dev_alloc<double>(h, sizeof(double) * (size_t)blocks_for(g.vs, 64), "allocate partials");
         h->scal = dev_alloc<CgScalars>(h, sizeof(CgScalars), "allocate CG state");
-        cuda_check(h, cudaMallocHost(reinterpret_cast<void**>(&h->scal_host), sizeof(CgScalars)),
+        // the CG state and, behind it, resident.cu's timeout flag
+        const size_t pinned = sizeof(CgScalars) + sizeof(int);
+        cuda_check(h, cudaHostAlloc(reinterpret_cast<void**>(&h->scal_host), pinned, cudaHostAllocMapped),
                    "allocate pinned CG state");
-        std::memset(h->scal_host, 0, sizeof(CgScalars));
+        std::memset(h->scal_host, 0, pinned);
         h->resident = resident_fits(g, false) || (h->opt.inner != STAG_INNER_NONE && resident_fits(g, true));
         if (h->resident) {
-            h->rwork.slots = dev_alloc<double>(h, sizeof(double) * 2 * kResidentMaxBlocks, "allocate exchange");
-            h->rwork.count = dev_alloc<unsigned int>(h, sizeof(unsigned int), "allocate exchange");
-            h->rwork.base = dev_alloc<unsigned int>(h, sizeof(unsigned int), "allocate exchange");
-            h->rwork.ns = dev_alloc<unsigned long long>(h, sizeof(unsigned long long) * STAG_KERNEL_COUNT,
-                                                        "allocate times");
-            cuda_check(h, cudaHostAlloc(reinterpret_cast<void**>(&h->timeout_host), sizeof(int), cudaHostAllocMapped),
-                       "allocate mapped flag");
-            *h->timeout_host = 0;
+            // one allocation: partial sums, phase times, the counter and its base
+            constexpr size_t slots = 2 * kResidentMaxBlocks, words = slots + STAG_KERNEL_COUNT + 1;
+            h->rwork.slots = dev_alloc<double>(h, sizeof(double) * words, "allocate exchange");
+            h->rwork.ns = reinterpret_cast<unsigned long long*>(h->rwork.slots + slots);
+            h->rwork.count = reinterpret_cast<unsigned int*>(h->rwork.ns + STAG_KERNEL_COUNT);
+            h->rwork.base = h->rwork.count + 1;
+            h->timeout_host = reinterpret_cast<int*>(h->scal_host + 1);
             cuda_check(h, cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->rwork.timeout), h->timeout_host, 0),
                        "map flag");
         }

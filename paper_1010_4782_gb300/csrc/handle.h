@@ -63,7 +63,7 @@ struct stag_handle {
     // small lattices: the iterations in one launch (resident.cu)
     bool resident = false;
     stag::ResidentWork rwork{nullptr, nullptr, nullptr, nullptr, nullptr};
-    int* timeout_host = nullptr;  // host-mapped: a bounded device-side wait ran out
+    int* timeout_host = nullptr;  // in scal_host's allocation: a bounded device-side wait ran out
     // graphs
     cudaGraphExec_t graph = nullptr;
     // timing
