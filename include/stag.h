@@ -176,6 +176,11 @@ int stag_set_stream(stag_handle* h, void* cuda_stream);
 /* Change m of Eq. (3); must be finite. */
 int stag_set_mass(stag_handle* h, double mass);
 
+/* Most polls (of about 0.5 us) of a wait between the blocks of the small lattices'
+ * launch before the call gives up with STAG_ERR_TIMEOUT; < 0: the default, about
+ * two seconds.  0: a block waits for no other (a test of the error). */
+int stag_set_wait_limit(stag_handle* h, int32_t polls);
+
 /* Half of D (Sec. 2, Eq. (5)): out = D_{P,1-P} in, i.e. D restricted to output
  * sites of parity P = out_parity (0 even, 1 odd) acting on a vector of parity
  * 1-P.  in, out: [V/2][3] complex128, must not overlap.  Native FP64 arithmetic
@@ -203,8 +208,9 @@ int stag_apply_A_prec(stag_handle* h, int32_t arith, const double* in_even, doub
  * the true residual is then recomputed with native FP64 arithmetic and Fig. 1
  * restarts from the current x while it exceeds tol (at most max_restarts times).
  * Returns STAG_OK, STAG_ERR_NOT_CONVERGED (x holds the last iterate) or
- * STAG_ERR_BREAKDOWN; info (nullable) is filled in every case.  (STAG_ERR_TIMEOUT: a
- * bounded wait between the blocks of the small lattices' launch ran out.) */
+ * STAG_ERR_BREAKDOWN; info (nullable) is filled in every case.  STAG_ERR_TIMEOUT: a
+ * bounded wait between the blocks of the small lattices' launch ran out; x_even is
+ * left as it was and the handle can be used as before. */
 int stag_cg_solve(stag_handle* h, const double* b_even, double* x_even, double tol,
                   int32_t max_iter, stag_solve_info* info);
 

@@ -56,6 +56,7 @@ EXPORTED = (
     "stag_create_ex",
     "stag_set_stream",
     "stag_set_mass",
+    "stag_set_wait_limit",
     "stag_dslash",
     "stag_apply_A",
     "stag_apply_A_prec",
@@ -170,6 +171,7 @@ def load(path: str | None = None):
                                    ctypes.POINTER(stag_options)]
     lib.stag_set_stream.argtypes = [H, P]
     lib.stag_set_mass.argtypes = [H, d]
+    lib.stag_set_wait_limit.argtypes = [H, i32]
     lib.stag_dslash.argtypes = [H, i32, P, P]
     lib.stag_apply_A.argtypes = [H, P, P]
     lib.stag_apply_A_prec.argtypes = [H, i32, P, P]
@@ -282,6 +284,10 @@ def stag_set_stream(h, stream):
 
 def stag_set_mass(h, mass):
     _check(load().stag_set_mass(h, float(mass)), h)
+
+
+def stag_set_wait_limit(h, polls):
+    _check(load().stag_set_wait_limit(h, int(polls)), h)
 
 
 def stag_dslash(h, out_parity, inp, out):

@@ -124,10 +124,17 @@ void begin_call(stag_handle* h) {
     cuda_check(h, cudaStreamWaitEvent(h->s, h->ev_in, 0), "cudaStreamWaitEvent");
 }
 
+// Phase times, and the counter and its base in one word, behind the partial sums.
+constexpr size_t kExchangeWords = STAG_KERNEL_COUNT + 1;
+
 void end_call(stag_handle* h) {
     cuda_check(h, cudaStreamSynchronize(h->s), "cudaStreamSynchronize");
     if (h->timeout_host && *static_cast<volatile int*>(h->timeout_host)) {
         *h->timeout_host = 0;
+        // the blocks left at different exchanges: the counter and its base start again
+        // (and the phase times in front of them)
+        cuda_check(h, cudaMemsetAsync(h->rwork.ns, 0, kExchangeWords * sizeof(double), h->s), "clear exchange");
+        cuda_check(h, cudaStreamSynchronize(h->s), "cudaStreamSynchronize");
         fail(h, STAG_ERR_TIMEOUT, "a bounded wait between the blocks of a kernel ran out");
     }
 }
@@ -895,8 +902,8 @@ int stag_create_ex(stag_handle** out, const double* fat, const double* naik_long
         h->resident = resident_fits(g, false) || (h->opt.inner != STAG_INNER_NONE && resident_fits(g, true));
         if (h->resident) {
             // one allocation: partial sums, phase times, the counter and its base
-            constexpr size_t slots = 2 * kResidentMaxBlocks, words = slots + STAG_KERNEL_COUNT + 1;
-            h->rwork.slots = dev_alloc<double>(h, sizeof(double) * words, "allocate exchange");
+            constexpr size_t slots = 2 * kResidentMaxBlocks;
+            h->rwork.slots = dev_alloc<double>(h, sizeof(double) * (slots + kExchangeWords), "allocate exchange");
             h->rwork.ns = reinterpret_cast<unsigned long long*>(h->rwork.slots + slots);
             h->rwork.count = reinterpret_cast<unsigned int*>(h->rwork.ns + STAG_KERNEL_COUNT);
             h->rwork.base = h->rwork.count + 1;
@@ -965,6 +972,12 @@ int stag_set_mass(stag_handle* h, double mass) {
         return STAG_ERR_INVALID_ARG;
     }
     h->mass = mass;
+    return STAG_OK;
+}
+
+int stag_set_wait_limit(stag_handle* h, int32_t polls) {
+    if (!h) return STAG_ERR_INVALID_ARG;
+    h->rwork.polls = polls < 0 ? kResidentPolls : polls;
     return STAG_OK;
 }
 

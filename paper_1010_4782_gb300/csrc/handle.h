@@ -62,7 +62,7 @@ struct stag_handle {
     stag::CgScalars* scal_host = nullptr;  // pinned
     // small lattices: the iterations in one launch (resident.cu)
     bool resident = false;
-    stag::ResidentWork rwork{nullptr, nullptr, nullptr, nullptr, nullptr};
+    stag::ResidentWork rwork;
     int* timeout_host = nullptr;  // in scal_host's allocation: a bounded device-side wait ran out
     // graphs
     cudaGraphExec_t graph = nullptr;

@@ -28,7 +28,8 @@
 // pipes above.
 //
 // Waits are bounded: a block that polls too long raises the timeout flag and
-// leaves, and the host reports STAG_ERR_TIMEOUT.
+// leaves, and the host reports STAG_ERR_TIMEOUT.  The blocks then left at different
+// exchanges, so the counter and its base agree no longer; the host clears both.
 #include <algorithm>
 #include <atomic>
 
@@ -38,17 +39,15 @@ namespace stag {
 
 namespace {
 
-constexpr int kPollLimit = 1 << 22;  // polls of about 0.5 us before a wait gives up
-
 // Adds one to *count, after everything the block stored, and waits (one thread)
-// until it has reached target; false if it does not within kPollLimit polls.
-__device__ __forceinline__ bool arrive_and_wait(unsigned int* count, unsigned int target) {
+// until it has reached target; false if it does not within `limit` polls.
+__device__ __forceinline__ bool arrive_and_wait(unsigned int* count, unsigned int target, int limit) {
     unsigned int v;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(count) : "memory");
     ++v;
     int polls = 0;
     while ((int)(v - target) < 0) {
-        if (++polls > kPollLimit) return false;
+        if (++polls > limit) return false;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
     }
     return true;
@@ -246,7 +245,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
             if (lane == 0) {
                 if (sum) slots[blk] = mine;
                 target += nblk;
-                failed = failed || !arrive_and_wait(p.w.count, target);
+                failed = failed || !arrive_and_wait(p.w.count, target, p.w.polls);
             }
             __syncwarp();
             double tot = 0.0;

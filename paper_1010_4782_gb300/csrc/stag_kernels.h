@@ -97,12 +97,14 @@ void launch_dslash_b16(const Geom& g, int out_parity, const __nv_bfloat162* fat,
 
 // ---- the iterations of Fig. 1 in one cooperative launch, small lattices (resident.cu)
 constexpr int kResidentMaxBlocks = 256;
+constexpr int kResidentPolls = 1 << 22;  // of about 0.5 us
 struct ResidentWork {
-    double* slots;           // [2][kResidentMaxBlocks]: the blocks' partial sums
-    unsigned int* count;     // arrivals so far, zero at first
-    unsigned int* base;      // their number when the last launch ended, zero at first
-    int* timeout;            // host-mapped, set to 1 when a bounded wait ran out
-    unsigned long long* ns;  // nullable: time of D_oe, D_eo, the x/r update and the d update, added up
+    double* slots = nullptr;           // [2][kResidentMaxBlocks]: the blocks' partial sums
+    unsigned int* count = nullptr;     // arrivals so far, zero at first and after a timeout
+    unsigned int* base = nullptr;      // count + 1: their number when the last launch ended, likewise
+    int* timeout = nullptr;            // host-mapped, set to 1 when a bounded wait ran out
+    unsigned long long* ns = nullptr;  // nullable: time of D_oe, D_eo, the x/r update and the d update, added up
+    int polls = kResidentPolls;        // of a wait before it gives up
 };
 // Does every site get a thread of its own at once?  (fp32: FP32 arithmetic)
 bool resident_fits(const Geom& g, bool fp32);
