@@ -101,7 +101,7 @@ typedef struct {
     int32_t max_restarts;   /* restarts of Fig. 1 from the current x when the true residual
                                exceeds tol (default 5)                                        */
     int32_t use_graphs;     /* capture check_interval iterations as one CUDA graph (default 1);
-                               no effect on those small lattices                               */
+                               no effect on those small lattices in one launch                 */
     int32_t timing;         /* record CUDA events around every CG kernel (default 0; on those
                                small lattices the device's clock around every phase of the
                                launch); disables graphs; read with stag_kernel_stats           */
@@ -175,6 +175,11 @@ int stag_set_stream(stag_handle* h, void* cuda_stream);
 
 /* Change m of Eq. (3); must be finite. */
 int stag_set_mass(stag_handle* h, double mass);
+
+/* The iterations of small lattices (see check_interval) in one launch of many (1, the
+ * default) or, as on a device that cannot hold its grid at once, in launches of four
+ * kernels each (0). */
+int stag_set_one_launch(stag_handle* h, int32_t enable);
 
 /* Most polls (of about 0.5 us) of a wait between the blocks of the small lattices'
  * launch before the call gives up with STAG_ERR_TIMEOUT; < 0: the default, about

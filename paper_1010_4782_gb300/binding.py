@@ -56,6 +56,7 @@ EXPORTED = (
     "stag_create_ex",
     "stag_set_stream",
     "stag_set_mass",
+    "stag_set_one_launch",
     "stag_set_wait_limit",
     "stag_dslash",
     "stag_apply_A",
@@ -171,6 +172,7 @@ def load(path: str | None = None):
                                    ctypes.POINTER(stag_options)]
     lib.stag_set_stream.argtypes = [H, P]
     lib.stag_set_mass.argtypes = [H, d]
+    lib.stag_set_one_launch.argtypes = [H, i32]
     lib.stag_set_wait_limit.argtypes = [H, i32]
     lib.stag_dslash.argtypes = [H, i32, P, P]
     lib.stag_apply_A.argtypes = [H, P, P]
@@ -284,6 +286,10 @@ def stag_set_stream(h, stream):
 
 def stag_set_mass(h, mass):
     _check(load().stag_set_mass(h, float(mass)), h)
+
+
+def stag_set_one_launch(h, enable):
+    _check(load().stag_set_one_launch(h, int(bool(enable))), h)
 
 
 def stag_set_wait_limit(h, polls):

@@ -329,13 +329,16 @@ constexpr int kResidentIters = 512;
 // Is the iteration's arithmetic FP32 (the mixed-precision inner iteration)?
 bool iterates_in_fp32(const stag_handle* h) { return h->opt.inner != STAG_INNER_NONE; }
 
-// False if the device cannot hold the grid at once (a context limited to some of the SMs).
+// False if the device cannot hold the grid at once (a context limited to some of the SMs),
+// or as if it could not (stag_set_one_launch).
 bool launch_resident(stag_handle* h, int iters) {
     const Geom& g = h->g;
     ResidentWork w = h->rwork;
     if (!h->opt.timing) w.ns = nullptr;
     cudaError_t e;
-    if (iterates_in_fp32(h)) {
+    if (!h->one_launch) {
+        e = cudaErrorCooperativeLaunchTooLarge;
+    } else if (iterates_in_fp32(h)) {
         LoLinks L;
         L.fat32 = h->fat32;
         L.lng32 = h->lng32;
@@ -372,7 +375,7 @@ bool run_fig1_resident(stag_handle* h) {
     long long iter_before = 0;  // a run starts at iteration 0
     do {
         if (!launch_resident(h, iters)) {
-            h->resident = false;
+            h->one_launch = false;
             return false;
         }
         read_state(h);
@@ -978,6 +981,12 @@ int stag_set_mass(stag_handle* h, double mass) {
 int stag_set_wait_limit(stag_handle* h, int32_t polls) {
     if (!h) return STAG_ERR_INVALID_ARG;
     h->rwork.polls = polls < 0 ? kResidentPolls : polls;
+    return STAG_OK;
+}
+
+int stag_set_one_launch(stag_handle* h, int32_t enable) {
+    if (!h) return STAG_ERR_INVALID_ARG;
+    h->one_launch = enable != 0;
     return STAG_OK;
 }
 

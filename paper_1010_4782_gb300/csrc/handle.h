@@ -61,7 +61,8 @@ struct stag_handle {
     stag::CgScalars* scal = nullptr;
     stag::CgScalars* scal_host = nullptr;  // pinned
     // small lattices: the iterations in one launch (resident.cu)
-    bool resident = false;
+    bool resident = false;   // the lattice is small enough
+    bool one_launch = true;  // false: not wanted, or the device could not hold the grid
     stag::ResidentWork rwork;
     int* timeout_host = nullptr;  // in scal_host's allocation: a bounded device-side wait ran out
     // graphs
