@@ -128,7 +128,7 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-DSLASH_SOURCES = ("dslash.cu", "dirac.cuh", "links.cuh", "ff.cuh", "stag_internal.cuh")
+DSLASH_SOURCES = ("dslash.cu", "dirac.cuh", "links.cuh", "ff.cuh", "ff_bits.h", "stag_internal.cuh")
 MULTI_SOURCES = ("multi.cu", "multi.cuh", "links.cuh", "stag_internal.cuh")
 
 

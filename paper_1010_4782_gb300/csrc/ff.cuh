@@ -18,69 +18,14 @@
 
 #include <cuda_runtime.h>
 
+#include "ff_bits.h"
 #include "stag_internal.cuh"
 
 namespace stag {
 
-// hi = fl32(a), lo = fl32(a - hi).  For exponents from 2^-70 to 2^120 by integer
-// arithmetic on a's bits, the same bits as the conversions give: those (and the
-// subtraction) run on the FP64 pipe at two lanes per cycle and SM, which bound the vector
-// conversions (32^3 x 64 on GB300: pack and unpack run in 19 and 20 us, 100 MB each).
 __device__ __forceinline__ float2 ff_from_double(double a) {
-    const int h = __double2hiint(a);
-    const unsigned int l = (unsigned int)__double2loint(a);
-    const int e = ((h >> 20) & 0x7ff) - 1023;
-    if (e < -70 || e > 120) {  // zero, tiny, huge, not finite
-        const float hi = __double2float_rn(a);
-        return make_float2(hi, __double2float_rn(a - (double)hi));
-    }
-    // significand: 24 bits q and 29 bits below them, rounded to nearest even
-    unsigned int q = ((unsigned int)(h & 0xfffff) << 3) | 0x800000u | (l >> 29);
-    int rem = (int)(l & 0x1fffffffu);
-    const bool up = rem > 0x10000000 || (rem == 0x10000000 && (q & 1u));
-    if (up) {
-        q += 1;
-        rem -= 0x20000000;
-    }
-    const unsigned int sign = (unsigned int)h & 0x80000000u;
-    if (sign) rem = -rem;
-    const float hi = __uint_as_float(sign | (((unsigned int)(e + 127) << 23) + (q - 0x800000u)));
-    const float lo = __fmul_rn(__int2float_rn(rem), __uint_as_float((unsigned int)(e - 52 + 127) << 23));
-    return make_float2(hi, lo);
-}
-
-// (double)hi + (double)lo, rounded to nearest even; by integer arithmetic as above where hi is
-// a normal number of ordinary size and lo below its last place.
-__device__ __forceinline__ double ff_sum(float hi, float lo) {
-    const unsigned int h = __float_as_uint(hi), l = __float_as_uint(lo);
-    const int eh = (int)((h >> 23) & 0xff), el = (int)((l >> 23) & 0xff);
-    const bool lo_zero = (l << 1) == 0u;
-    if (eh < 40 || eh > 250 || !(lo_zero || (el >= 1 && eh - el >= 23))) return (double)hi + (double)lo;
-    // 24-bit significands; hi's leading bit at 61, lo's bits below the shift kept as a sticky one
-    unsigned long long s = (unsigned long long)((h & 0x7fffffu) | 0x800000u) << 38;
-    if (!lo_zero) {
-        const unsigned long long m = (l & 0x7fffffu) | 0x800000u;
-        const int shift = 38 - (eh - el);
-        unsigned long long t;
-        if (shift >= 0)
-            t = m << shift;
-        else if (shift > -24)
-            t = (m >> -shift) | ((m & ((1ull << -shift) - 1ull)) != 0ull);
-        else
-            t = 1ull;
-        s = ((h ^ l) & 0x80000000u) ? s - t : s + t;
-    }
-    int e = eh - 127;
-    if (!(s >> 61)) {
-        s <<= 1;
-        e -= 1;
-    }
-    unsigned long long q = s >> 9;
-    const unsigned int rem = (unsigned int)s & 0x1ffu;
-    q += rem > 0x100u || (rem == 0x100u && (q & 1ull));
-    const unsigned long long bits = ((unsigned long long)(h & 0x80000000u) << 32) |
-                                    (((unsigned long long)(e + 1023) << 52) + (q - (1ull << 52)));
-    return __longlong_as_double((long long)bits);
+    const FFPair p = ff_split(a);
+    return make_float2(p.hi, p.lo);
 }
 
 // complex float-float in one 16-byte word: (re_hi, re_lo, im_hi, im_lo)
