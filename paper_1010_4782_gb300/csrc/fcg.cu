@@ -87,11 +87,17 @@ struct Arith<double2> {
     static __device__ __forceinline__ float2 f2(double2 v) { return make_float2((float)v.x, (float)v.y); }
 };
 
-// A block's sum (thread 0).  Float-float values stay float-float, as wide as the threads'
-// sums: FP64 adds run at two lanes per cycle and SM, and the shuffles' two FP64 sums took
-// 10 of fcg_out_kernel's 48 us at 24^3 x 48.
-__device__ __forceinline__ double block_total(double v, double* sm) { return block_sum<kBlock>(v, sm); }
-__device__ __forceinline__ double block_total(FFAcc v, double*) { return block_sum<kBlock>(v); }
+// A block's sums of a and b in FP64 (thread 0).
+__device__ __forceinline__ void block_totals(double a, double b, double (&sum)[2]) {
+    __shared__ double sm[kBlock / 32];
+    sum[0] = block_sum<kBlock>(a, sm);
+    __syncthreads();
+    sum[1] = block_sum<kBlock>(b, sm);
+}
+__device__ __forceinline__ void block_totals(FFAcc a, FFAcc b, double (&sum)[2]) {
+    const FFAcc v[2] = {a, b};
+    block_sums<kBlock>(v, sum);
+}
 
 // Two grid sums at once: per-block partials of a and b, then the last block to
 // finish adds them in block order (deterministic).  True in every thread of
@@ -102,12 +108,11 @@ __device__ __forceinline__ bool grid_sum2_last_block(Acc va, Acc vb, double* par
     __shared__ double sm[kBlock / 32];
     __shared__ bool is_last;
     __shared__ double res[2];
-    const double a = block_total(va, sm);
-    __syncthreads();
-    const double b = block_total(vb, sm);
+    double sum[2];
+    block_totals(va, vb, sum);
     if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = a;
-        partials[2 * blockIdx.x + 1] = b;
+        partials[2 * blockIdx.x] = sum[0];
+        partials[2 * blockIdx.x + 1] = sum[1];
         __threadfence();
         is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
@@ -263,7 +268,7 @@ __global__ void __launch_bounds__(kBlock) fcg_zdots_kernel(Geom g, const T* __re
 // sites (pt_out_site; chi from pt_chi_kernel), stored in FP32, with (z, r),
 // (z, q) and beta as in fcg_zdots_kernel.  Latency-bound like pt_chi_kernel: the eight
 // directions unrolled and three blocks an SM (80 registers) 52 -> 46 us at 24^3 x 48, the
-// float-float block sums 38 us (167 MB: 25 us at measured HBM rate); the solve there 129.2 -> 121.4 ms.
+// block sums off the FP64 pipe 39 us (167 MB: 25 us at measured HBM rate); the solve there 129.2 -> 122.3 ms.
 template <class V, class TS, class L>
 __global__ void __launch_bounds__(kBlock, 3) fcg_out_kernel(Geom g, const L* __restrict__ links,
                                                          const float2* __restrict__ coef, const TS* __restrict__ chi,

@@ -86,20 +86,39 @@ __device__ __forceinline__ float2 ff_result(const FFAcc& a) {
     return make_float2(hi, lo);
 }
 
-__device__ __forceinline__ double ff_acc_to_double(const FFAcc& a) {
-    return (double)a.s + (double)a.e;
-}
+// A warp's sum in 64-bit fixed point (ff_bits.h): the sums of the 27-bit parts of its
+// numbers, or, where one of them is not finite (E = 255), the bits of the sum in FP64.
+struct alignas(16) FixedSum {
+    unsigned int lo, mid;
+    int hi, E;
+};
 
-// Sum over the warp, in every lane (fixed tree).
-__device__ __forceinline__ FFAcc ff_warp_sum(FFAcc a) {
+// Sum of a over the warp, in every lane: each number is rounded once, to 2^-57 of the
+// largest one's binade at the worst (an FP64 tree rounds every partial sum), and the
+// integer reduction instructions add them.
+__device__ __forceinline__ FixedSum ff_warp_sum(FFAcc a) {
+    const unsigned int all = 0xffffffffu;
+    FixedSum f;
+    f.E = (int)__reduce_max_sync(all, (unsigned int)max(float_exponent(a.s), float_exponent(a.e)));
+    if (f.E == 255) {
+        double v = (double)a.s + (double)a.e;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        FFAcc x;
-        x.s = __shfl_xor_sync(0xffffffffu, a.s, o);
-        x.e = __shfl_xor_sync(0xffffffffu, a.e, o);
-        ff_merge(a, x);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(all, v, o);
+        f.lo = (unsigned int)__double2loint(v);
+        f.mid = (unsigned int)__double2hiint(v);
+        f.hi = 0;
+        return f;
     }
-    return a;
+    const long long v = float_to_fixed(a.s, f.E) + float_to_fixed(a.e, f.E);
+    const unsigned int part = (1u << 27) - 1u;
+    f.lo = __reduce_add_sync(all, (unsigned int)v & part);
+    f.mid = __reduce_add_sync(all, (unsigned int)(v >> 27) & part);
+    f.hi = (int)__reduce_add_sync(all, (unsigned int)(int)(v >> 54));
+    return f;
+}
+__device__ __forceinline__ double sum_value(const FixedSum& f) {
+    if (f.E == 255) return __hiloint2double((int)f.mid, (int)f.lo);
+    return fixed_to_double((long long)f.lo + ((long long)f.mid << 27) + ((long long)f.hi << 54), f.E);
 }
 
 // One row of a 3x3 complex product for one hop, accumulated locally and
@@ -211,23 +230,39 @@ __device__ __forceinline__ void ff_redot_acc(FFAcc& acc, float4 a, float4 b) {
     ff_mac(acc, a.z, a.w, b.z, b.w);
 }
 
-// Sum of v over the block in float-float additions, in FP64, valid in thread 0 (relative
-// rounding 2^-48 of the block's sum, against 2^-24 or 2^-48 in the values themselves).
-// The FP64 pipe takes 16 cycles for one addition of a warp: the 45 of a 256-thread
-// block's tree slowed the reducing D_eo of 28^3 x 96 by 2 to 4 us.
+// Sums of N values over the block in FP64, valid in thread 0 (fixed tree).  The FP64 pipe
+// takes 16 cycles for one operation of a warp, and shuffle trees in every warp, with the
+// conversions before them, are 67 of them in a block of 256 threads; here it is the
+// three additions of the warps' sums.  Rounding, rms over blocks of 256 norms: 6.4e-17
+// (FP64 trees 7.3e-17, float-float trees 2.5e-15).  The float-float D_eo of 28^3 x 96
+// takes 419 us, 422 with one warp adding 256 FP64 values, 417 with float-float trees.
+template <int BS, int N>
+__device__ __forceinline__ void block_sums(const FFAcc (&v)[N], double (&sum)[N]) {
+    constexpr int NW = BS / 32;
+    static_assert(N * NW <= 32, "one warp adds them");
+    __shared__ FixedSum warps[N * NW];
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const FixedSum f = ff_warp_sum(v[k]);
+        if (lane == 0) warps[k * NW + (threadIdx.x >> 5)] = f;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double s = lane < N * NW ? sum_value(warps[lane]) : 0.0;
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+    for (int k = 0; k < N; ++k) sum[k] = k ? __shfl_sync(0xffffffffu, s, k * NW) : s;
+}
 template <int BS>
 __device__ __forceinline__ double block_sum(FFAcc v) {
-    __shared__ float2 warps[BS / 32];
-    v = ff_warp_sum(v);
-    if ((threadIdx.x & 31) == 0) warps[threadIdx.x >> 5] = make_float2(v.s, v.e);
-    __syncthreads();
-    if (threadIdx.x != 0) return 0.0;
-    FFAcc a{warps[0].x, warps[0].y};
-#pragma unroll
-    for (int w = 1; w < BS / 32; ++w) ff_merge(a, FFAcc{warps[w].x, warps[w].y});
-    return ff_acc_to_double(a);
+    const FFAcc in[1] = {v};
+    double sum[1] = {0.0};
+    block_sums<BS>(in, sum);
+    return sum[0];
 }
-// grid_sum_last_block with the block's sum as above; the sum over blocks is FP64.
+// grid_sum_last_block with the block's sum as above.
 template <int BS>
 __device__ __forceinline__ bool grid_sum_last_block(FFAcc v, double* partials, unsigned int* counter, double* total) {
     return grid_total_last_block<BS>(block_sum<BS>(v), partials, counter, total);

@@ -88,4 +88,44 @@ STAG_BITS_FN double ff_sum(float hi, float lo) {
     return bits_as<double>(bits);
 }
 
+// ---- sums of FP32 numbers in 64-bit fixed point
+// The unit is 2^-56 of 2^(E - 127), E the largest biased exponent of the numbers added: a
+// number is below 2^57 units and exact unless it is more than 2^33 times smaller than
+// the largest.
+STAG_BITS_FN int float_exponent(float x) {  // biased; 1 for zero and subnormals
+    const int e = (int)((bits_as<unsigned int>(x) >> 23) & 0xffu);
+    return e ? e : 1;
+}
+
+// x in units, rounded to nearest (E >= float_exponent(x), x finite).
+STAG_BITS_FN long long float_to_fixed(float x, int E) {
+    const unsigned int b = bits_as<unsigned int>(x);
+    const unsigned int m = (b & 0x7fffffu) | ((b & 0x7f800000u) ? 0x800000u : 0u);
+    const int shift = 33 - (E - float_exponent(x));
+    long long v = 0;
+    if (shift >= 0)
+        v = (long long)((unsigned long long)m << shift);
+    else if (shift >= -24)
+        v = (long long)((m + (1u << (-shift - 1))) >> -shift);
+    return (b >> 31) ? -v : v;
+}
+
+// v units in FP64, rounded to nearest even.
+STAG_BITS_FN double fixed_to_double(long long v, int E) {
+    if (v == 0) return 0.0;
+    const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ull;
+    const unsigned long long u = sign ? 0ull - (unsigned long long)v : (unsigned long long)v;
+#if defined(__CUDA_ARCH__)
+    const int lz = __clzll((long long)u);
+#else
+    const int lz = __builtin_clzll(u);
+#endif
+    const unsigned long long n = u << lz;  // leading bit at 63
+    unsigned long long q = n >> 11;
+    const unsigned int rem = (unsigned int)n & 0x7ffu;
+    q += rem > 0x400u || (rem == 0x400u && (q & 1ull));
+    const int e = 63 - lz + E - (127 + 56);
+    return bits_as<double>(sign | (((unsigned long long)(e + 1023) << 52) + (q - (1ull << 52))));
+}
+
 }  // namespace stag

@@ -20,9 +20,9 @@
 // every block adds the blocks' partial sums in block order, so that the sum,
 // alpha, beta and the decision to stop are the same bits in every block.
 //
-// Per iteration, before (four launches in a graph) and now: 4^4 one-hop FP64 38 -> 14.6
-// us, 8^3 x 16 float-float 50 -> 15.2, FP64 91 -> 23.5, 16^4 one-hop FP32 26 -> 17.6,
-// 20 x 18 x 14 x 30 FP32 43 -> 32.5 (solve times over iterations, reliable updates
+// Per iteration, before (four launches in a graph) and now: 4^4 one-hop FP64 38 -> 14.2
+// us, 8^3 x 16 float-float 50 -> 15.3, FP64 91 -> 23.3, 16^4 one-hop FP32 26 -> 17.6,
+// 20 x 18 x 14 x 30 FP32 43 -> 32.8 (solve times over iterations, reliable updates
 // included), 16^3 x 32 float-float 104 -> 66.  Bound now: the exchanges and the FP64
 // scalars below 10,000 sites (about 9 us of an iteration), L2 and the FP32 or FP64
 // pipes above.
@@ -61,14 +61,13 @@ __device__ __forceinline__ unsigned long long now_ns() {
 
 // -------------------------------------------- the vector steps, per arithmetic
 // Own: r and d as stored; X: the solution's increment (float-float, FP32) or the
-// solution (FP64); Sum: a thread's or warp's part of a dot product.
-__device__ __forceinline__ FFAcc warp_sum(FFAcc s) { return ff_warp_sum(s); }
+// solution (FP64); Sum: a thread's part of a dot product.
 __device__ __forceinline__ double warp_sum(double s) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
 }
-__device__ __forceinline__ double sum_value(FFAcc s) { return ff_acc_to_double(s); }
+
 __device__ __forceinline__ double sum_value(double s) { return s; }
 
 struct StepScalars {
@@ -186,7 +185,10 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
     constexpr int NS = 32 / S;
     constexpr bool kFF = std::is_same<A, ArithFF>::value;
     if (p.scal->done) return;
-    __shared__ double s_part[32];
+    // parts of a dot product, added by one warp: of every warp (FP32 types), or of every site
+    // (FP64: the pipe takes 16 cycles for an addition of a warp, so no tree in every warp)
+    constexpr bool kWarpSums = std::is_same<typename Ops::Sum, FFAcc>::value;
+    __shared__ typename std::conditional<kWarpSums, FixedSum, double>::type s_val[THREADS / (kWarpSums ? 32 : S)];
     __shared__ StepScalars s_step;
     __shared__ CgScalars s_sc;
     __shared__ unsigned long long s_ns[4], s_t0;
@@ -228,17 +230,25 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
     unsigned int n_exchange = 0;
     bool failed = false;  // (thread 0)
 
-    // Publishes the sum over the block's warps of v (sum = true) and waits for every
-    // block; thread 0 then runs finish(total).
-    auto exchange = [&](bool sum, double v, auto finish) {
+    // Publishes the sum over the block's sites of v (sum = true) in FP64 and waits for
+    // every block; thread 0 then runs finish(total).
+    auto exchange = [&](bool sum, typename Ops::Sum v, auto finish) {
         ++n_exchange;
-        if (sum && lane == 0) s_part[warp] = v;
+        if (sum) {
+            if constexpr (kWarpSums) {
+                const FixedSum w = ff_warp_sum(v);
+                if (lane == 0) s_val[warp] = w;
+            } else if (part == 0) {
+                s_val[warp * NS + lane] = v;
+            }
+        }
         __syncthreads();
         if (warp == 0) {
             double mine = 0.0;
             if (sum) {
-                mine = lane < nwarp ? s_part[lane] : 0.0;
-                mine = warp_sum(mine);
+                const int n = kWarpSums ? nwarp : nwarp * NS;
+                for (int k = lane; k < n; k += 32) mine += sum_value(s_val[k]);
+                for (int o = 1; o < n && o < 32; o <<= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
             }
             // two sets of slots in turn: a block is at most one exchange ahead of the slowest
             double* const slots = p.w.slots + (n_exchange & 1u) * kResidentMaxBlocks;
@@ -295,7 +305,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
                 for (int c = 0; c < 3; ++c) p.t[c * vs + i] = A::store_val(acc, c);
             }
         }
-        exchange(false, 0.0, [](double) {});
+        exchange(false, Ops::zero(), [](double) {});
         lap(0);
         if (s_step.stop) break;
         typename Ops::Sum s = Ops::zero();
@@ -308,8 +318,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
                 s = A::dot(acc);
             }
         }
-        s = warp_sum(s);
-        exchange(true, lane == 0 ? sum_value(s) : 0.0, [&](double total) {
+        exchange(true, s, [&](double total) {
             sc.pAp = total;
             sc.alpha = sc.delta_new / total;
             if (!(total > 0.0) || !isfinite(sc.alpha)) {
@@ -326,8 +335,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
         if (s_step.stop) break;
         s = Ops::zero();
         if (own) Ops::update_xr(s_step, d, ad, x, r, s);
-        s = warp_sum(s);
-        exchange(true, lane == 0 ? sum_value(s) : 0.0, [&](double total) {
+        exchange(true, s, [&](double total) {
             sc.delta_old = sc.delta_new;
             sc.delta_new = total;
             sc.beta = total / sc.delta_old;
@@ -363,7 +371,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const ResidentPara
             }
         }
         if (it == p.iters) break;
-        exchange(false, 0.0, [](double) {});
+        exchange(false, Ops::zero(), [](double) {});
         lap(3);
         if (s_step.stop) break;
     }

@@ -13,9 +13,21 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1010_4782_gb300", "csrc")
 SHIM = """
+#include <initializer_list>
 #include "ff_bits.h"
 extern "C" void sums(const float* hi, const float* lo, double* out, long n) {
     for (long k = 0; k < n; ++k) out[k] = stag::ff_sum(hi[k], lo[k]);
+}
+extern "C" void fixed_sums(const float* s, const float* e, double* out, long n) {  // of 32 pairs each
+    for (long k = 0; k < n / 32; ++k) {
+        int E = 1;
+        for (long j = 32 * k; j < 32 * k + 32; ++j)
+            for (float x : {s[j], e[j]})
+                if (stag::float_exponent(x) > E) E = stag::float_exponent(x);
+        long long v = 0;
+        for (long j = 32 * k; j < 32 * k + 32; ++j) v += stag::float_to_fixed(s[j], E) + stag::float_to_fixed(e[j], E);
+        out[k] = stag::fixed_to_double(v, E);
+    }
 }
 extern "C" void splits(const double* a, float* hi, float* lo, long n) {
     for (long k = 0; k < n; ++k) {
@@ -92,3 +104,33 @@ def test_split(shim, e):
         l = (a - h.astype(np.float64)).astype(np.float32)
     for got, want in ((hi, h), (lo, l)):
         assert ((got.view(np.uint32) == want.view(np.uint32)) | (np.isnan(got) & np.isnan(want))).all()
+
+
+@pytest.mark.parametrize("spread", [0, 3, 30, 33, 34, 60, 250])
+@pytest.mark.parametrize("top", [1, 2, 60, 127, 200, 254])
+def test_fixed_point_sum_of_a_warp(shim, top, spread):
+    """32 pairs (s, e): exact, then rounded once, when every number is within 2^33 of the
+    largest; else each is rounded to 2^-57 of the largest's binade.  Against Fractions; an
+    FP64 tree of the same numbers is allowed to be no better in the worst case."""
+    from fractions import Fraction
+    rng = np.random.default_rng(1000 * top + spread)
+    groups = 60
+    ex = np.clip(top - rng.integers(0, spread + 1, (groups, 32)), 0, 254).astype(np.uint32)
+    ex[:, 0] = top
+    s = (ex << np.uint32(23)) | rng.integers(0, 1 << 23, (groups, 32), dtype=np.uint32)
+    s[::3] |= rng.integers(0, 2, (len(s[::3]), 32), dtype=np.uint32) << np.uint32(31)  # signs; the others positive
+    s[1, 1:] = 0
+    s[2] = np.uint32((top << 23) | 0x7FFFFF)   # the largest sum
+    s = s.view(np.float32)
+    e = (s * rng.uniform(-2.0 ** -23, 2.0 ** -23, s.shape)).astype(np.float32)
+    e[2] = s[2]
+    out = np.empty(s.size)
+    _call(shim.fixed_sums, s.ravel().copy(), e.ravel().copy(), out)
+    unit = Fraction(2) ** (top - 127 - 56)
+    for k in range(groups):
+        numbers = [Fraction(float(v)) for v in (*s[k], *e[k])]
+        exact = sum(numbers)
+        near = all(v == 0 or abs(v) >= unit * 2 ** 23 for v in numbers)
+        slack = Fraction(0) if near else 64 * unit / 2
+        got = Fraction(float(out[k]))
+        assert abs(got - exact) <= slack + abs(exact) * Fraction(1, 2 ** 53) * Fraction(1001, 1000)
