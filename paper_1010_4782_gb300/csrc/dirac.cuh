@@ -102,7 +102,6 @@ struct ArithF32 {
     using TL = T;  // link storage
     static constexpr int kEntries = 9;  // stored entries per link
     static constexpr bool kRecon = false;
-    static __device__ __forceinline__ C ldl(const TL* p) { return ld(p); }
     struct Acc {
         float2 c[3];
         float dot;
@@ -142,7 +141,6 @@ struct ArithH16 {
     using TL = T;  // link storage
     static constexpr int kEntries = 9;  // stored entries per link
     static constexpr bool kRecon = false;
-    static __device__ __forceinline__ C ldl(const TL* p) { return ld(p); }
     using Acc = ArithF32::Acc;
     using Sum = ArithF32::Sum;
     static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
@@ -168,7 +166,6 @@ struct ArithB16 {
     using TL = T;  // link storage
     static constexpr int kEntries = 9;  // stored entries per link
     static constexpr bool kRecon = false;
-    static __device__ __forceinline__ C ldl(const TL* p) { return ld(p); }
     using Acc = ArithF32::Acc;
     using Sum = ArithF32::Sum;
     static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
@@ -196,7 +193,6 @@ struct ArithF32R {
     static constexpr int kEntries = 6;
     static constexpr bool kRecon = true;
     static __device__ __forceinline__ C ld(const T* p) { return __ldg(p); }
-    static __device__ __forceinline__ C ldl(const TL* p) { return __ldg(p); }
     using Acc = ArithF32::Acc;
     using Sum = ArithF32::Sum;
     static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }
@@ -222,7 +218,6 @@ struct ArithL16 {
     static constexpr bool kRecon = false;
     using C = float2;
     static __device__ __forceinline__ C ld(const T* p) { return __ldg(p); }
-    static __device__ __forceinline__ C ldl(const TL* p) { return __half22float2(__ldg(p)); }
     using Acc = ArithF32::Acc;
     using Sum = ArithF32::Sum;
     static __device__ __forceinline__ Sum dot(const Acc& a) { return ArithF32::dot(a); }

@@ -31,9 +31,10 @@ namespace stag {
 
 // Resident 256-thread blocks per SM the register allocation is held to.  The
 // float-float kernels are bound by memory latency: with up to 128 registers
-// (2 blocks) the compiler keeps more of a site's loads in flight, and the
-// float-float CG solve at 28^3 x 96 measured 1304 ms against 1320 ms with 3
-// blocks (80 registers), 1339 ms with 4 (64) and 1734 ms with 1.  The others
+// (2 blocks) the compiler keeps more of a site's loads in flight, and a
+// float-float CG solve of 665 iterations at 28^3 x 96 takes 598 ms against 630 ms
+// with 3 blocks (80 registers), 677 ms with 4 (64) and 798 ms with 1.  (At 24^3 x 48, 483
+// iterations, 3 blocks are ahead: 153 ms, 159 with 2, 194 with 4, 200 with 1.)  The others
 // keep 4 blocks (64 registers; 3 and 80 with two-row Naik links): FP64 is
 // bound by its pipe and FP32 by HBM, where more registers measured no gain.
 template <class A, int NAIK>

@@ -190,12 +190,6 @@ __device__ __forceinline__ float2 ff_renorm(float s, float e) {
     return make_float2(hi, lo);
 }
 
-__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
-    float err;
-    const float s = two_sum(a.x, b.x, err);
-    return ff_renorm(s, __fadd_rn(err, __fadd_rn(a.y, b.y)));
-}
-
 // a * b + c
 __device__ __forceinline__ float2 ff_fma(float2 a, float2 b, float2 c) {
     const FFAcc p = ff_prod(a.x, a.y, b.x, b.y);
@@ -205,8 +199,6 @@ __device__ __forceinline__ float2 ff_fma(float2 a, float2 b, float2 c) {
 }
 
 __device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
-
-__device__ __forceinline__ double ff_to_double(float2 a) { return (double)a.x + (double)a.y; }
 
 // complex helpers on (re_hi, re_lo, im_hi, im_lo)
 __device__ __forceinline__ float2 ff_re(float4 a) { return make_float2(a.x, a.y); }

@@ -398,24 +398,6 @@ __global__ void __launch_bounds__(kBlock) pt_dot_f32_kernel(Geom g, const float2
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
-// |v|^2 of an even-site vector (T, [3][vs]) -> per-block partials (FP64)
-template <class T>
-__global__ void __launch_bounds__(kBlock) pt_norm2_kernel(Geom g, const T* __restrict__ v, double* partials) {
-    const int i = blockIdx.x * kBlock + threadIdx.x;
-    const size_t vs = (size_t)g.vs;
-    double acc = 0.0;
-    if (i < g.vh) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float2 a = ldc(v + c * vs + i);
-            acc += (double)a.x * a.x + (double)a.y * a.y;
-        }
-    }
-    __shared__ double sm[kBlock / 32];
-    const double s = block_sum<kBlock>(acc, sm);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
 // slot (T, even [3][vs]) = scale * v, v an FP64 or float-float SoA vector
 template <class TS, class T>
 __global__ void __launch_bounds__(kBlock) pt_store_slot_kernel(Geom g, const TS* __restrict__ v, double scale,
@@ -813,12 +795,6 @@ double slot_energy(stag_ptnet* n, const void* slot) {
     apply_A_f32(n);
     pt_dot_f32_kernel<<<blocks_for(g.vh), kBlock, 0, S(n)>>>(g, n->vad, n->vad, n->red);
     return read_partials(n, blocks_for(g.vh));
-}
-
-template <class T>
-double slot_norm2(stag_ptnet* n, const void* slot) {
-    pt_norm2_kernel<T><<<blocks_for(n->g.vh), kBlock, 0, S(n)>>>(n->g, static_cast<const T*>(slot), n->red);
-    return read_partials(n, blocks_for(n->g.vh));
 }
 
 // forward through all layers from act[0]

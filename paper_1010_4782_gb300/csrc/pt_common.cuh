@@ -74,10 +74,6 @@ __device__ __forceinline__ void st4c(float2* p, float2 v0, float2 v1, float2 v2,
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-// conj(a) * b
-__device__ __forceinline__ float2 cmulf_conj(float2 a, float2 b) {
-    return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
 
 __device__ __forceinline__ int pt_neighbour(const Geom& g, int x, int y, int z, int t, int mu, bool up) {
     switch (mu) {

@@ -88,8 +88,6 @@ __device__ __forceinline__ int wrap_dn(int c, int k, int L) {
 }
 
 // ------------------------------------------------------- FP64 complex ops
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-
 // acc += a * b
 __device__ __forceinline__ void cmac(double2& acc, double2 a, double2 b) {
     acc.x = fma(a.x, b.x, acc.x);
