@@ -97,7 +97,9 @@ typedef struct {
     int32_t check_interval; /* CG iterations between host convergence reads (default 32); lattices
                                small enough for one launch of many iterations (up to about
                                78,000 sites of a parity in FP64 class, 156,000 in FP32) read
-                               every 512 rounded down to a multiple of it                     */
+                               every 512 rounded down to a multiple of it, or every
+                               check_interval if that is more (one kernel then holds the
+                               device for up to 0.7 s, at 4096)                               */
     int32_t max_restarts;   /* restarts of Fig. 1 from the current x when the true residual
                                exceeds tol (default 5)                                        */
     int32_t use_graphs;     /* capture check_interval iterations as one CUDA graph (default 1);

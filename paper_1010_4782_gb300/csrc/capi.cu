@@ -4,7 +4,7 @@
 // The driver keeps alpha, beta and delta on the device (the paper's CUBLAS
 // dot returned a scalar to the host every step).  It enqueues blocks of
 // check_interval iterations - captured once as a CUDA graph, or for small
-// lattices up to 512 of them in one cooperative launch (resident.cu) - and reads
+// lattices some 512 of them in one cooperative launch (resident.cu) - and reads
 // the CG state back only between blocks.  After Fig. 1 stops, the true residual
 // b - A x is recomputed with native FP64 arithmetic and Fig. 1 restarts from
 // the current x while it exceeds tol.
@@ -322,8 +322,8 @@ void ensure_graph(stag_handle* h) {
     cuda_check(h, e, "graph instantiate");
 }
 
-// Most iterations of one launch of resident.cu (a few milliseconds, so that a
-// call never holds the GPU for long in one kernel).
+// Iterations of one launch of resident.cu, rounded down to a multiple of check_interval (5 to
+// 85 ms at 10 to 165 us an iteration); a larger check_interval is one launch.
 constexpr int kResidentIters = 512;
 
 // Is the iteration's arithmetic FP32 (the mixed-precision inner iteration)?

@@ -8,8 +8,9 @@
 // 16-bit, nine entries: two words and one 4-byte plane).  One load per word instead
 // of one per entry: a warp reads 512 contiguous bytes where an FP16 entry plane gave it
 // 128, with 3 loads and 3 addresses per link instead of 9.  At 28^3 x 96 (Naik) the
-// D_oe with FP16 storage went from 102 to 94 us (0.99 of measured HBM); the FP32 ones stayed at
-// HBM speed (181 us, 156 us with two-row Naik links).  Where the links come from L2 fewer
+// D_oe with FP16 storage went from 102 to 93 us (632 MB: the rate of a plain copy, 0.91 to 0.93
+// of the 7.3 to 7.5 TB/s that a plain read sweep reaches); the FP32 ones stayed at HBM
+// speed (181 us, 156 us with two-row Naik links).  Where the links come from L2 fewer
 // loads show: 24^2 x 16 x 32 FP32 28.3 -> 25.3 us, 12^3 x 16 4.4 -> 3.3 us.
 // FP64 and float-float entries are 16-byte words themselves.
 #pragma once

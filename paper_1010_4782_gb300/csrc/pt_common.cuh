@@ -17,7 +17,7 @@ constexpr int kPaths = 9;
 constexpr int kHidden = 8;
 constexpr int kLayers = 3;
 constexpr int kChan[kLayers + 1] = {1, kHidden, kHidden, 1};
-constexpr int kWgradWave = 4 * 2 * 152;          // blocks of a weight-gradient launch: four waves of two per SM
+constexpr int kWgradWave = 4 * 2 * 152;          // blocks of a weight-gradient launch: four waves of two on each of GB300's 152 SMs
 constexpr int kWgradBlocks = kWgradWave / 9;      // most x-blocks of one (all nine paths)
 
 __device__ __forceinline__ float2 ldc(const float2* p) { return *p; }
