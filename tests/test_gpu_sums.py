@@ -58,3 +58,23 @@ def test_flexible_cg_of_a_large_source(form):
             B.stag_ptnet_destroy(net)
 
     _pair((10, 6, 4, 12), 2.0 ** 61, solve)
+
+
+@pytest.mark.parametrize("inner", [B.STAG_INNER_NONE, B.STAG_INNER_F32])
+@pytest.mark.parametrize("dims,one_launch", [((10, 6, 4, 12), 0), ((10, 6, 4, 12), 1), ((24, 24, 16, 32), 1)],
+                         ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
+def test_sites_beyond_the_range_are_a_breakdown(dims, one_launch, inner):
+    """With a site's own |r|^2 beyond the FP32 range the sums are infinite or NaN, and the solve
+    ends as a breakdown; the handle's next solve gives the bits of the one before."""
+    opt = B.stag_default_options()
+    opt.arith, opt.inner = B.STAG_ARITH_FF, inner
+    fat = torch.from_numpy(inputs.gauge_field(dims, 31)).cuda()
+    b = torch.from_numpy(inputs.gaussian_even_source(dims, 32)).cuda()
+    with B.Handle(fat, dims, MASS, options=opt) as h:
+        B.stag_set_one_launch(h.h, one_launch)
+        xs = []
+        for s, want in ((1.0, B.STAG_OK), (2.0 ** 66, B.STAG_ERR_BREAKDOWN), (1.0, B.STAG_OK)):
+            x = torch.zeros_like(b)
+            assert B.stag_cg_solve(h.h, s * b, x, TOL, 20000, raise_on_error=False)[0] == want
+            xs.append(x)
+    assert torch.equal(xs[0], xs[2])
